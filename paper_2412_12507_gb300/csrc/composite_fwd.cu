@@ -2,111 +2,190 @@
 // (Sec. 4.2, eq. GaussianMaxResponse; eq. QuadratureVolumeRendering) for a batch of views.
 // Each block leaves its tile's list as soon as every pixel's transmittance has dropped below
 // t_min; tiles run longest predicted walk first (k_fwd_predict + k_tile_order).
-#include "composite_common.cuh"
+#include "composite_warp.cuh"
 
 namespace ut3d {
 namespace {
 
+// Shared memory of one warp: its pixels' bounds and up to kRoundF staged survivors.
+constexpr int kRoundF = 32;
+
+template <int NST>
+struct __align__(16) FwdWarp {
+  WarpRays rays;
+  float4 geo[kRoundF][4];       // stage_particle's record
+  float col[kRoundF * NST];     // SH coefficients, or the colour (PP)
+  uint32_t idx[kRoundF], pos[kRoundF];  // particle, list position
+};
+
+// Resident blocks of 128 threads per SM that the kernel is compiled for.  Bound by issue and by the
+// latency of a chunk's loads, so more warps pay until the pixels' state spills.  Measured per call:
+// degree 3 on the 1M rolling-shutter 1080p view 1172 us a frame at 4 blocks (128 registers),
+// 1203 at 5, 1290 at 6; per-particle colours (no SH basis in registers) composite_forward of 200k
+// particles at 3840x2160 932 us at 5 blocks, 876 at 6, 831 at 8, but with a rolling shutter
+// 1104 us a frame at 5, 1095 at 6, 1170 at 8; degree 0 and 1 within 2 % from 5 to 8.
+constexpr int fwd_blocks(int deg, bool rs, bool pp) { return pp ? (rs ? 6 : 8) : (deg < 2 ? 6 : 4); }
+
+// Forward compositing, two pixels a thread and 64 a warp (composite_warp.cuh).  Against one pixel a
+// thread with the block's shared staging (1M rolling-shutter 1080p, k_composite_fwd alone): 578 M
+// -> 384 M warp instructions, 616 -> 507 us; composite_forward of 200k particles at 3840x2160
+// 1010 -> 835 us; the image is bit-identical.
+
 // PP: per-particle colour mode (the colour of each staged particle is evaluated once, at its
 // view direction, while staging; pixels read it from shared memory).
 template <int DEG, bool RS, bool STATS, bool PP, bool GEN>
-__global__ void __launch_bounds__(512) k_composite_fwd(const __grid_constant__ BatchDesc bd, DevOpts op,
-                                                       const short4 *__restrict__ rect,
-                                                       const uint32_t *__restrict__ vals,
-                                                       const uint2 *__restrict__ ranges,
-                                                       unsigned long long *__restrict__ stats, TileSched ts) {
+__global__ void __launch_bounds__(32 * kBlockWarps, fwd_blocks(DEG, RS, PP)) k_composite_fwd(const __grid_constant__ BatchDesc bd, DevOpts op,
+                                                          const short4 *__restrict__ rect,
+                                                          const uint32_t *__restrict__ vals,
+                                                          const uint2 *__restrict__ ranges,
+                                                          unsigned long long *__restrict__ stats, TileSched ts) {
   constexpr int NSH = (DEG + 1) * (DEG + 1);
   constexpr int NC = NSH * 3;
   constexpr int PDEG = PP ? 0 : DEG;        // per-pixel SH basis only when colours are per pixel
+  constexpr int PSH = (PDEG + 1) * (PDEG + 1);
   constexpr int NST = PP ? 4 : NC;          // staged colour floats per particle
-  __shared__ float4 s_geo[kBatchF][4];
-  __shared__ __align__(16) float s_sh[kBatchF * NST];
-  __shared__ uint32_t s_idx[kBatchF];
+  extern __shared__ __align__(16) unsigned char smem[];
 
   // tiles in the order k_tile_order gave them (longest predicted walk first); every tile is
   // in the order, so every pixel is written
-  if (blockIdx.x >= *ts.n_work) return;
-  const int tile = (int)ts.order[blockIdx.x];
+  const uint32_t rank = blockIdx.x / (uint32_t)tile_blocks(op);
+  if (rank >= *ts.n_work) return;
+  const int tile = (int)ts.order[rank];
   UT_DBG_CHECK(tile < bd.total_tiles, UT_DBG_TILE_ID, tile, bd.total_tiles, 2);
   const DevView &view = bd.v[view_of_tile(bd, tile)];
   const DevScene &sc = bd.s[view.scene];
   const DevCam &cam = view.cam;
+  const int lane = threadIdx.x & 31;
+  const int warp = (int)(blockIdx.x % (uint32_t)tile_blocks(op)) * kBlockWarps + (int)(threadIdx.x >> 5);  // of the tile
+  if (warp >= tile_warps(op)) return;  // warps never wait for each other
+  FwdWarp<NST> &S = reinterpret_cast<FwdWarp<NST> *>(smem)[threadIdx.x >> 5];
   const int lt = tile - view.tile_off;
-  const int tx = lt % view.tiles_x, ty = lt / view.tiles_x;
-  int lx, ly;
-  tile_pixel(op, (int)threadIdx.x, lx, ly);
-  const int px = tx * op.tile_w + lx;
-  const int py = ty * op.tile_h + ly;
-  const bool inside = px < cam.W && py < cam.H;
-  float3 o, d;
-  float Y[(PDEG + 1) * (PDEG + 1)];
-  bool valid;
-  pixel_setup<PDEG>(cam, op, px, py, inside, o, d, Y, valid);
+  const int x0 = (lt % view.tiles_x) * op.tile_w, y0 = (lt / view.tiles_x) * op.tile_h;
 
-  float T = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f;
-  uint32_t last = 0;
-  unsigned long long n_eval = 0, n_blend = 0;
-  bool done = !valid;
-  const uint2 rg = ranges[tile];
-  for (uint32_t start = rg.x; start < rg.y; start += kBatchF) {
-    if (__syncthreads_count(!done) == 0) break;
-    const int nb = min((uint32_t)kBatchF, rg.y - start);
-    for (int t = threadIdx.x; t < nb; t += blockDim.x) s_idx[t] = vals[start + t];
-    __syncthreads();
-    for (int t = threadIdx.x; t < nb; t += blockDim.x) {
-      uint32_t idx = s_idx[t];
-      stage_particle<RS>(sc, cam, op, rect[view.part_off + idx], idx, s_geo[t], nullptr);
-      if (PP) reinterpret_cast<float4 *>(s_sh)[t] = particle_colour<DEG, RS>(sc, cam, op, idx);
-    }
-    if (!PP) stage_sh<NC>(sc, s_idx, nb, s_sh);
-    __syncthreads();
-    if (done) continue;
-    for (int b = 0; b < nb; ++b) {
-      float3 og, dg;
-      float dd, a;
-      if (STATS) {
-        int r0 = __float_as_int(s_geo[b][3].z), r1 = __float_as_int(s_geo[b][3].w);
-        n_eval += !(px < (r0 & 0xffff) || px > (r1 & 0xffff) || py < (r0 >> 16) || py > (r1 >> 16));
-      }
-      if (!eval_response<RS, GEN>(s_geo[b], px, py, o, d, og, dg, dd, a, op)) continue;
-      float al = fminf(a, op.alpha_max);
-      float Tn = T * (1.f - al);
-      if (Tn < op.t_min) {
-        done = true;
-        break;
-      }
-      if (STATS) ++n_blend;
-      float r0, r1, r2;
-      if (PP) {
-        const float4 c = reinterpret_cast<const float4 *>(s_sh)[b];
-        r0 = c.x; r1 = c.y; r2 = c.z;
-      } else {
-        sh_colour<NSH>(s_sh + b * NC, Y, r0, r1, r2);
-      }
-      float w = al * T;
-      C0 = fmaf(fmaxf(r0, 0.f), w, C0);
-      C1 = fmaf(fmaxf(r1, 0.f), w, C1);
-      C2 = fmaf(fmaxf(r2, 0.f), w, C2);
-      T = Tn;
-      last = start + b + 1;
-    }
+  f3x2 o, d;
+  float2 Y[PSH];
+  uint32_t pk[2];  // the pixels still walking, kDead once stopped
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    int lx, ly;
+    const bool in = tile_pixel2(op, warp, lane, h, lx, ly);
+    const int px = x0 + lx, py = y0 + ly;
+    float3 oh, dh;
+    float Yh[PSH];
+    bool valid;
+    pixel_setup<PDEG>(cam, op, px, py, in && px < cam.W && py < cam.H, oh, dh, Yh, valid);
+    pk[h] = valid ? (uint32_t)px | ((uint32_t)py << 16) : kDead;
+    (h ? o.x.y : o.x.x) = oh.x; (h ? o.y.y : o.y.x) = oh.y; (h ? o.z.y : o.z.x) = oh.z;
+    (h ? d.x.y : d.x.x) = dh.x; (h ? d.y.y : d.y.x) = dh.y; (h ? d.z.y : d.z.x) = dh.z;
+#pragma unroll
+    for (int k = 0; k < PSH; ++k) (h ? Y[k].y : Y[k].x) = Yh[k];
   }
-  if (inside) {
-    size_t pix = (size_t)py * cam.W + px;
-    size_t plane = (size_t)cam.W * cam.H;
-    view.rgb[pix] = C0;
-    view.rgb[plane + pix] = C1;
-    view.rgb[2 * plane + pix] = C2;
-    view.alpha[pix] = valid ? 1.f - T : 0.f;
-    if (view.tfinal) view.tfinal[pix] = T;
-    if (view.n_used) view.n_used[pix] = last;
+  warp_rays(pk, o, d, tile_is_8x8(op), lane, &S.rays);
+  __syncwarp();
+
+  float T[2] = {1.f, 1.f}, C[2][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
+  uint32_t last[2] = {0u, 0u};
+  unsigned long long n_eval = 0, n_blend = 0;
+  const uint2 rg = ranges[tile];
+  // entries of this chunk of 32 and of the next one (their rectangles are loaded a chunk ahead)
+  uint32_t idx = list_index(vals, rg.x + lane, rg.y), idx1 = list_index(vals, rg.x + 32 + lane, rg.y);
+  short4 r = list_rect(rect, view.part_off, idx, rg.x + lane, rg.y);
+  for (uint32_t p0 = rg.x; p0 < rg.y; p0 += 32) {
+    if (__all_sync(kFull, pk[0] == kDead && pk[1] == kDead)) break;
+    const short4 r1 = list_rect(rect, view.part_off, idx1, p0 + 32 + lane, rg.y);
+    const uint32_t idx2 = list_index(vals, p0 + 64 + lane, rg.y);
+    bool near_ = rect_near(S.rays, r);
+    float4 g[4];
+    if (near_) {
+      stage_particle<RS>(sc, cam, op, r, idx, g, nullptr);
+      near_ = !block_misses<RS>(g, S.rays) || STATS;  // the counting variant walks every rectangle
+    }
+    const unsigned m = __ballot_sync(kFull, near_);
+    const int n = __popc(m);
+    if (near_) {
+      const int b = __popc(m & ((1u << lane) - 1u));
+#pragma unroll
+      for (int q = 0; q < 4; ++q) S.geo[b][q] = g[q];
+      S.idx[b] = idx;
+      S.pos[b] = p0 + lane;
+      if (PP) reinterpret_cast<float4 *>(S.col)[b] = particle_colour<DEG, RS>(sc, cam, op, idx);
+    }
+    __syncwarp();
+    if (!PP) stage_sh_warp<NC>(sc, S.idx, n, S.col, lane);
+    int bl[2] = {-1, -1};  // last survivor blended by each pixel
+    for (int b = 0; b < n; ++b) {
+      const float4 g3 = S.geo[b][3];
+      const uint32_t r0 = __float_as_uint(g3.z), re = __float_as_uint(g3.w);
+      bool h0 = in_rect(pk[0], r0, re), h1 = in_rect(pk[1], r0, re);
+      if (STATS) n_eval += (int)h0 + (int)h1;
+      if (!(h0 || h1)) continue;
+      const PairEval e = eval_pair<RS>(S.geo[b][0], S.geo[b][1], S.geo[b][2], o, d);
+      h0 = h0 && e.cc.x <= g3.y * e.dd.x;
+      h1 = h1 && e.cc.y <= g3.y * e.dd.y;
+      if (!(h0 || h1)) continue;
+      const float al0 = fminf(response<GEN>(g3.x, e.cc.x, e.dd.x, op), op.alpha_max);
+      const float al1 = fminf(response<GEN>(g3.x, e.cc.y, e.dd.y, op), op.alpha_max);
+      const float Tn0 = T[0] * (1.f - al0), Tn1 = T[1] * (1.f - al1);
+      if (h0 && Tn0 < op.t_min) {
+        pk[0] = kDead;
+        h0 = false;
+      }
+      if (h1 && Tn1 < op.t_min) {
+        pk[1] = kDead;
+        h1 = false;
+      }
+      if (STATS) n_blend += (int)h0 + (int)h1;
+      float2 c0, c1, c2;
+      if (PP) {
+        const float4 c = reinterpret_cast<const float4 *>(S.col)[b];
+        c0 = bc(c.x); c1 = bc(c.y); c2 = bc(c.z);
+      } else {
+        sh_colour2<NSH>(S.col + b * NC, Y, c0, c1, c2);
+      }
+      if (h0) {
+        const float w = al0 * T[0];
+        C[0][0] = fmaf(fmaxf(c0.x, 0.f), w, C[0][0]);
+        C[0][1] = fmaf(fmaxf(c1.x, 0.f), w, C[0][1]);
+        C[0][2] = fmaf(fmaxf(c2.x, 0.f), w, C[0][2]);
+        T[0] = Tn0;
+        bl[0] = b;
+      }
+      if (h1) {
+        const float w = al1 * T[1];
+        C[1][0] = fmaf(fmaxf(c0.y, 0.f), w, C[1][0]);
+        C[1][1] = fmaf(fmaxf(c1.y, 0.f), w, C[1][1]);
+        C[1][2] = fmaf(fmaxf(c2.y, 0.f), w, C[1][2]);
+        T[1] = Tn1;
+        bl[1] = b;
+      }
+    }
+    if (bl[0] >= 0) last[0] = S.pos[bl[0]] + 1;
+    if (bl[1] >= 0) last[1] = S.pos[bl[1]] + 1;
+    __syncwarp();  // the survivors are read before the next chunk's are staged
+    idx = idx1;
+    idx1 = idx2;
+    r = r1;
+  }
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    int lx, ly;
+    const bool in = tile_pixel2(op, warp, lane, h, lx, ly);
+    const int px = x0 + lx, py = y0 + ly;
+    if (!in || px >= cam.W || py >= cam.H) continue;
+    const size_t pix = (size_t)py * cam.W + px, plane = (size_t)cam.W * cam.H;
+    view.rgb[pix] = C[h][0];
+    view.rgb[plane + pix] = C[h][1];
+    view.rgb[2 * plane + pix] = C[h][2];
+    view.alpha[pix] = 1.f - T[h];  // 0 where the pixel has no ray: T stays 1
+    if (view.tfinal) view.tfinal[pix] = T[h];
+    if (view.n_used) view.n_used[pix] = last[h];
   }
   if (STATS) {
     for (int s = 16; s >= 1; s >>= 1) {
-      n_eval += __shfl_xor_sync(0xffffffffu, n_eval, s);
-      n_blend += __shfl_xor_sync(0xffffffffu, n_blend, s);
+      n_eval += __shfl_xor_sync(kFull, n_eval, s);
+      n_blend += __shfl_xor_sync(kFull, n_blend, s);
     }
-    if ((threadIdx.x & 31) == 0) {
+    if (lane == 0) {
       atomicAdd(&stats[0], n_eval);
       atomicAdd(&stats[1], n_blend);
     }
@@ -294,16 +373,24 @@ __global__ void k_fwd_predict(const __grid_constant__ BatchDesc bd, DevOpts op, 
   }
 }
 
+template <int DEG, bool RS, bool STATS, bool PP, bool GEN>
+void fwd_launch_s(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, const uint32_t *vals,
+                  const uint32_t *ranges, unsigned long long *stats, const TileSched &ts, cudaStream_t s) {
+  constexpr int NST = PP ? 4 : 3 * (DEG + 1) * (DEG + 1);
+  const int warps = block_warps(op);
+  const size_t smem = sizeof(FwdWarp<NST>) * (size_t)warps;
+  if (smem > 48 * 1024)
+    cudaFuncSetAttribute(k_composite_fwd<DEG, RS, STATS, PP, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem);
+  k_composite_fwd<DEG, RS, STATS, PP, GEN><<<bd.total_tiles * tile_blocks(op), 32 * warps, smem, s>>>(
+      bd, op, reinterpret_cast<const short4 *>(rect), vals, reinterpret_cast<const uint2 *>(ranges), stats, ts);
+}
+
 template <int DEG, bool RS, bool PP, bool GEN>
 void fwd_launch_k(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, const uint32_t *vals,
                   const uint32_t *ranges, unsigned long long *stats, const TileSched &ts, cudaStream_t s) {
-  const int blocks = bd.total_tiles, threads = op.tile_w * op.tile_h;
-  const short4 *r4 = reinterpret_cast<const short4 *>(rect);
-  const uint2 *rg = reinterpret_cast<const uint2 *>(ranges);
-  if (stats)
-    k_composite_fwd<DEG, RS, true, PP, GEN><<<blocks, threads, 0, s>>>(bd, op, r4, vals, rg, stats, ts);
-  else
-    k_composite_fwd<DEG, RS, false, PP, GEN><<<blocks, threads, 0, s>>>(bd, op, r4, vals, rg, nullptr, ts);
+  if (stats) fwd_launch_s<DEG, RS, true, PP, GEN>(bd, op, rect, vals, ranges, stats, ts, s);
+  else fwd_launch_s<DEG, RS, false, PP, GEN>(bd, op, rect, vals, ranges, stats, ts, s);
 }
 
 // Degree 0 colours do not depend on the direction: both colour modes run the per-pixel kernel.
