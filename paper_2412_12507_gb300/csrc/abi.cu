@@ -220,6 +220,9 @@ ut_status check_scene(const ut_scene *s, bool need_sh) {
 
 bool aligned8(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 7u) == 0; }
 
+// Every particle's row of SH values is 16-byte aligned.
+int rows_aligned16(const float *sh, int deg) { return (3 * (deg + 1) * (deg + 1)) % 4 == 0 && aligned16(sh); }
+
 DevScene scene_desc(const ut_scene &s) {
   DevScene d;
   std::memset(&d, 0, sizeof(d));
@@ -230,8 +233,7 @@ DevScene scene_desc(const ut_scene &s) {
   d.sh = s.sh;
   d.n = s.n;
   d.deg = s.sh_degree;
-  const int nc = 3 * (s.sh_degree + 1) * (s.sh_degree + 1);
-  d.sh_vec = (nc % 4 == 0) && aligned16(s.sh);
+  d.sh_vec = rows_aligned16(s.sh, s.sh_degree);
   return d;
 }
 
@@ -584,6 +586,7 @@ ut_status composite_backward(const ut_scene *scene, const ut_camera *cam, const 
   s.d_quats = d_quats;
   s.d_logits = d_opacity_logits;
   s.d_sh = d_sh;
+  s.dsh_vec = rows_aligned16(d_sh, scene->sh_degree);
   s.grad_off = 0;
   return launch_composite_bwd(bd, dop, rect, vals, tile_ranges, static_cast<char *>(workspace) + acc_bytes,
                               reinterpret_cast<cudaStream_t>(stream));
@@ -669,6 +672,7 @@ ut_status render_batch_backward(const ut_scene *scenes, int32_t n_scenes, const 
     s.d_quats = g.d_quats;
     s.d_logits = g.d_opacity_logits;
     s.d_sh = g.d_sh;
+    s.dsh_vec = rows_aligned16(g.d_sh, scenes[k].sh_degree);
     s.grad_off = goff;
     goff += scenes[k].n;
   }

@@ -5,13 +5,13 @@
 // suffix sums S_i = C - sum_{j<=i} c_j alpha_j T_j without dividing transmittances,
 // and n_used tells each pixel where the forward stopped.  Per (particle, warp) the 13
 // geometry partials are reduced with a transposing reduce-scatter and the 3 x (deg+1)^2 SH
-// partials with a tensor-core contraction over the warp's pixels; both are accumulated
-// across warps in shared memory and pushed to global memory with one atomic per value per
-// (tile, particle).  A final per-particle kernel maps the accumulated dL/dM, dL/dmu,
-// dL/dsigma onto log-scales, quaternions and logits.  Tiles run heaviest replay first.
+// partials with a tensor-core contraction over the warp's pixels; both go to the particle's
+// accumulators in global memory as coalesced reductions.  A final per-particle kernel maps the
+// accumulated dL/dM, dL/dmu, dL/dsigma onto log-scales, quaternions and logits.  Tiles run
+// heaviest replay first.
 #include <cuda_bf16.h>
 
-#include "composite_common.cuh"
+#include "composite_warp.cuh"
 
 namespace ut3d {
 namespace {
@@ -51,305 +51,368 @@ __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], 
 }
 
 constexpr int kSlots = 8;     // particle columns of one tensor-core flush (the MMA's N)
+constexpr int kRoundB = 24;   // survivors staged at a time: 17 KB a warp, 12 warps an SM
 
-// Float index of (row, col) in a warp's 32-column W tile: columns are XOR-swizzled by the row so
-// that the fragment loads of four rows (8-byte pairs, 16 lanes per phase) hit distinct banks
-// without padding.
-__device__ __forceinline__ int wtile(int row, int col) { return row * 32 + (col ^ ((row & 3) << 3)); }
-
-// Shared-memory layout of the backward kernel (dynamic; bytes for a block of `warps` warps).
-// PP: per-particle colour mode (no SH coefficients staged, no W tiles).
+// Shared memory of one warp of the backward.
 template <int DEG, bool PP>
-struct BwdSmem {
+struct __align__(16) BwdWarp {
   static constexpr int NSH = (DEG + 1) * (DEG + 1);
   static constexpr int NC = NSH * 3;
-  static constexpr int NST = PP ? 4 : NC;                   // staged colour floats per particle
-  static constexpr int ACC = PP ? 17 : (16 + NC) | 1;      // accumulators per particle (odd: rows spread over banks)
-  static __host__ __device__ size_t geo() { return 0; }
-  static __host__ __device__ size_t aux() { return geo() + sizeof(float4) * 4 * kBatch; }
-  static __host__ __device__ size_t sh() { return aux() + sizeof(float4) * kBatch; }
-  static __host__ __device__ size_t acc() { return sh() + sizeof(float) * ((kBatch * NST + 3) / 4 * 4); }
-  static __host__ __device__ size_t wmat() { return acc() + sizeof(float) * kBatch * ACC; }
-  // per warp: 3 channels x kSlots rows of W (the first 16 rows double as the staging area of
-  // Y), then the A fragments (uint4 [4][32]: hi/lo of both k-steps, lane-minor)
-  static constexpr int kWRows = PP ? 0 : (3 * kSlots > 16 ? 3 * kSlots : 16);
-  static constexpr int kWarpFloats = PP ? 0 : kWRows * 32 + 4 * 4 * 32;
-  static __host__ __device__ size_t idx(int warps) { return wmat() + sizeof(float) * warps * kWarpFloats; }
-  static __host__ __device__ size_t any(int warps) { return idx(warps) + sizeof(uint32_t) * kBatch; }
-  static __host__ __device__ size_t bytes(int warps) { return any(warps) + sizeof(int) * kBatch; }
+  static constexpr int ROWS = PP ? 1 : (NSH > 8 ? 16 : 8);  // basis rows of the MMA's A that can be non-zero
+  static constexpr int COLS = PP ? 1 : 3 * kSlots;
+  // gradient rows on their way out: stride 60 for the 48 floats of degree 3 keeps the fragment
+  // writes free of bank conflicts, any multiple of 4 the 16-byte reads aligned
+  static constexpr int OST = NC == 48 ? 60 : (NC % 4 == 0 ? NC + 4 : NC);
+  WarpRays rays;
+  float4 geo[kRoundB][5];                   // stage_particle's record; o - mu or mu, list position
+  float col[kRoundB * (PP ? 4 : NC)];       // SH coefficients, or the colour (PP)
+  uint32_t idx[kRoundB];
+  uint32_t cidx[kSlots > kRoundB ? kSlots : kRoundB];  // particle of each column / outgoing row
+  float dc[PP ? kRoundB : 1][3];            // PP: dL/dcolour of every survivor
+  uint2 A[ROWS][32];                        // basis of the pixel pairs, (hi, lo) bf16 pairs
+  union {
+    uint2 W[COLS][32];                      // SH weights of the pixel pairs, row = channel x column
+    float out[(PP ? kRoundB : kSlots) * OST];
+  };
 };
 
-// Backward of k_composite_fwd for one tile.  Per (pixel, particle) pair the partials are
-// dL/dbeta_k,c = w_c Y_k (w_c = dL/dc_c alpha T where the colour is not clamped), the 9
-// products v x^T for dL/dM, v for dL/dmu and dL/dsigma.
+// Slot of pixel pair l in row `row` of A or W: the fragment loads read four consecutive pairs of
+// eight rows, which the XOR spreads over all banks.
+__device__ __forceinline__ int pair_slot(int row, int l) { return l ^ ((row & 7) << 2); }
+
+// Adds n gradient rows of NC floats (row b at out + b * stride, particle idx[b]) to d_sh: 16-byte
+// vector reductions when the rows are aligned, consecutive scalars otherwise (both coalesced; the
+// L2 takes 1.3 T float reductions a second that way against 0.13 T scattered ones).
+template <int NC>
+__device__ __forceinline__ void add_rows(const DevScene &sc, const float *out, int stride, const uint32_t *idx, int n,
+                                         int lane) {
+  if (NC % 4 == 0 && sc.dsh_vec) {
+    constexpr int N4 = NC % 4 == 0 ? NC / 4 : 1;
+    for (int f = lane; f < n * N4; f += 32) {
+      const int b = f / N4, j = 4 * (f - b * N4);
+      const float4 v = *reinterpret_cast<const float4 *>(out + b * stride + j);
+      asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(sc.d_sh + (size_t)idx[b] * NC + j), "f"(v.x),
+                   "f"(v.y), "f"(v.z), "f"(v.w)
+                   : "memory");
+    }
+  } else {
+    for (int f = lane; f < n * NC; f += 32) {
+      const int b = f / NC, j = f - b * NC;
+      atomicAdd(sc.d_sh + (size_t)idx[b] * NC + j, out[b * stride + j]);
+    }
+  }
+}
+
+// Backward of k_composite_fwd for one tile, walked like the forward (composite_warp.cuh): two
+// pixels a thread, survivors of the warp's own culling, no block barrier.  Per (pixel, particle)
+// pair the partials are dL/dbeta_k,c = w_c Y_k (w_c = dL/dc_c alpha T where the colour is not
+// clamped), the 9 products v x^T for dL/dM, v for dL/dmu and dL/dsigma.
 //
-// The SH part is a dense contraction over the warp's 32 pixels, D[k][j] = sum_p Y_k(p) W_c(p, j),
+// The SH part is a dense contraction over the warp's 64 pixels, D[k][j] = sum_p Y_k(p) W_c(p, j),
 // run on the tensor cores (m16n8k16, BF16 hi/lo split with the three cross terms, FP32
-// accumulate): A = Y^T (basis x pixels) is fixed for the tile and its fragments are parked in
-// shared memory; B = W (pixels x particles) collects, column by column, only particles that
-// reach at least one pixel of the warp, and is contracted once kSlots columns are full (and at
-// the end of each staged batch).  The 13 geometry partials are summed with a 16-value
-// reduce-scatter.  Both land in per-particle shared accumulators that are added to global
-// memory once per (tile, particle).
+// accumulate): A = Y^T (basis x pixels) is fixed for the tile; B = W (pixels x particles)
+// collects, column by column, only particles that reach at least one pixel of the warp, and is
+// contracted once kSlots columns are full.  A lane's two pixels are neighbours in the
+// contraction's order, so each lane splits and stores its own pair.  The 13 geometry partials are
+// summed over the pair, then with a 16-value reduce-scatter.  Both go straight to the particle's
+// accumulators in global memory with coalesced reductions, which the L2 absorbs (about 20 G rows
+// of 64 floats a second): no accumulators shared by the tile's warps, no flush, no barrier.
+// Bound by instruction issue (59 % of the cycles at 12 warps an SM).  Compiled for 3 blocks of 128
+// threads per SM (168 registers): at 4 blocks the pair's state spills (1M rolling-shutter 1080p
+// training step 2558 us against 2520, backward of 200k particles at 640x480 890 against 780), at 5
+// far more.  Against one pixel a thread with accumulators shared by the tile's warps: that step
+// 3112 -> 2520 us, that backward 1223 -> 780 us, the 8-view step of 3M particles 58.9 -> 46.3 ms
+// (with the forward's change).
 // PP (per-particle colour mode): the colour gradient dL/dc is one 3-vector per particle, summed
-// in the three spare slots of the reduce-scatter; at the per-(tile, particle) flush it becomes
+// in the three spare slots of the reduce-scatter; after each round it becomes
 // dL/dbeta = dL/dc Y(dir) and the mean's gradient through the view direction.
-// SMALL: tiles of at most 256 pixels, compiled for three resident blocks per SM (80 registers).
-template <int DEG, bool RS, bool SMALL, bool PP, bool GEN>
-__global__ void __launch_bounds__(SMALL ? 256 : 512, SMALL ? 3 : 1)
-    k_composite_bwd(const __grid_constant__ BatchDesc bd, DevOpts op,
-                                                       const short4 *__restrict__ rect,
-                                                       const uint32_t *__restrict__ vals,
-                                                       const uint2 *__restrict__ ranges, TileSched ts) {
-  using L = BwdSmem<DEG, PP>;
+template <int DEG, bool RS, bool PP, bool GEN>
+__global__ void __launch_bounds__(32 * kBlockWarps, 3) k_composite_bwd(const __grid_constant__ BatchDesc bd, DevOpts op,
+                                                          const short4 *__restrict__ rect,
+                                                          const uint32_t *__restrict__ vals,
+                                                          const uint2 *__restrict__ ranges, TileSched ts) {
+  using L = BwdWarp<DEG, PP>;
   constexpr int NSH = L::NSH;
   constexpr int NC = L::NC;
   constexpr int PDEG = PP ? 0 : DEG;  // per-pixel SH basis only when colours are per pixel
-  constexpr int ACC = L::ACC;
+  constexpr int PSH = (PDEG + 1) * (PDEG + 1);
   extern __shared__ __align__(16) unsigned char smem[];
-  const int warps = blockDim.x >> 5;
-  float4(*s_geo)[4] = reinterpret_cast<float4(*)[4]>(smem + L::geo());
-  float4 *s_aux = reinterpret_cast<float4 *>(smem + L::aux());
-  float *s_sh = reinterpret_cast<float *>(smem + L::sh());
-  float *s_acc = reinterpret_cast<float *>(smem + L::acc());
-  uint32_t *s_idx = reinterpret_cast<uint32_t *>(smem + L::idx(warps));
-  int *s_any = reinterpret_cast<int *>(smem + L::any(warps));
 
   // tiles in the order k_tile_order gave them (most list entries to replay first)
-  if (blockIdx.x >= *ts.n_work) return;
-  const int tile = (int)ts.order[blockIdx.x];
+  const uint32_t rank = blockIdx.x / (uint32_t)tile_blocks(op);
+  if (rank >= *ts.n_work) return;
+  const int tile = (int)ts.order[rank];
   UT_DBG_CHECK(tile < bd.total_tiles, UT_DBG_TILE_ID, tile, bd.total_tiles, 3);
   const DevView &view = bd.v[view_of_tile(bd, tile)];
   const DevScene &sc = bd.s[view.scene];
   const DevCam &cam = view.cam;
-  const int lt = tile - view.tile_off;
-  const int tx = lt % view.tiles_x, ty = lt / view.tiles_x;
-  int lx, ly;
-  tile_pixel(op, (int)threadIdx.x, lx, ly);
-  const int px = tx * op.tile_w + lx;
-  const int py = ty * op.tile_h + ly;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
+  const int warp = (int)(blockIdx.x % (uint32_t)tile_blocks(op)) * kBlockWarps + (int)(threadIdx.x >> 5);  // of the tile
+  if (warp >= tile_warps(op)) return;  // warps never wait for each other
   const int g8 = lane >> 2, t4 = lane & 3;
-  float *s_W = reinterpret_cast<float *>(smem + L::wmat()) + (size_t)warp * L::kWarpFloats;
-  uint4 *s_Af = reinterpret_cast<uint4 *>(s_W + L::kWRows * 32);
-  const bool inside = px < cam.W && py < cam.H;
-  float3 o, d;
-  float Y[(PDEG + 1) * (PDEG + 1)];
-  bool valid;
-  pixel_setup<PDEG>(cam, op, px, py, inside, o, d, Y, valid);
-
-  if constexpr (!PP) {
-  // A operand (basis x pixels), fixed for the whole tile: the warp's Y transposed through
-  // its W tile (row k = basis function k, column = lane), split into hi + lo fragments and
-  // parked in shared memory (s_Af[2 ks + 0] = hi, s_Af[2 ks + 1] = lo)
-#pragma unroll
-  for (int k = 0; k < 16; ++k) s_W[wtile(k, lane)] = k < NSH ? Y[k < NSH ? k : 0] : 0.f;
-  __syncwarp();
-#pragma unroll
-  for (int ks = 0; ks < 2; ++ks) {
-    const int c0 = 16 * ks + 2 * t4;
-    uint4 hi, lo;
-    split_bf16x2(s_W[wtile(g8, c0)], s_W[wtile(g8, c0 + 1)], hi.x, lo.x);
-    split_bf16x2(s_W[wtile(g8 + 8, c0)], s_W[wtile(g8 + 8, c0 + 1)], hi.y, lo.y);
-    split_bf16x2(s_W[wtile(g8, c0 + 8)], s_W[wtile(g8, c0 + 9)], hi.z, lo.z);
-    split_bf16x2(s_W[wtile(g8 + 8, c0 + 8)], s_W[wtile(g8 + 8, c0 + 9)], hi.w, lo.w);
-    s_Af[(2 * ks) * 32 + lane] = hi;
-    s_Af[(2 * ks + 1) * 32 + lane] = lo;
-  }
-  __syncwarp();
-  // W starts finite: unused columns of a partial flush only feed their own (discarded) outputs
-#pragma unroll
-  for (int r = 0; r < 3 * kSlots; ++r) s_W[wtile(r, lane)] = 0.f;
-  }
-
+  L &S = reinterpret_cast<L *>(smem)[threadIdx.x >> 5];
+  const int lt = tile - view.tile_off;
+  const int x0 = (lt % view.tiles_x) * op.tile_w, y0 = (lt / view.tiles_x) * op.tile_h;
   const uint2 rg = ranges[tile];
-  uint32_t my_end = 0;
-  float g0 = 0.f, g1 = 0.f, g2 = 0.f, gAT = 0.f, Cf0 = 0.f, Cf1 = 0.f, Cf2 = 0.f;  // gAT = dL/dalpha T_final
-  if (valid) {
-    size_t pix = (size_t)py * cam.W + px;
-    size_t plane = (size_t)cam.W * cam.H;
-    my_end = view.n_used[pix];
-    g0 = view.d_rgb[pix]; g1 = view.d_rgb[plane + pix]; g2 = view.d_rgb[2 * plane + pix];
-    gAT = view.d_alpha[pix] * view.tfinal[pix];
-    Cf0 = view.rgb[pix]; Cf1 = view.rgb[plane + pix]; Cf2 = view.rgb[2 * plane + pix];
-  }
-  const uint32_t block_end = rg.x + ts.work[tile];
-  uint32_t warp_end = my_end;  // no pixel of this warp blends a particle at or after warp_end
-#pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) warp_end = max(warp_end, __shfl_xor_sync(0xffffffffu, warp_end, o));
 
-  // Contracts the first `cols` columns of W with Y and adds them to the particles' SH
-  // accumulators; lane s < kSlots holds in slot_b the batch index of column s.
-  int slot_b = 0;
+  f3x2 o, d;
+  float2 Y[PSH];
+  uint32_t pk[2], end[2];  // the pixels with something to replay (kDead: none), and where each stops
+  float2 gr[3], Hf;  // upstream g = dL/drgb, and g . (composited colour) - dL/dalpha T_final
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    int lx, ly;
+    const bool in = tile_pixel2(op, warp, lane, h, lx, ly);
+    const int px = x0 + lx, py = y0 + ly;
+    float3 oh, dh;
+    float Yh[PSH];
+    bool valid;
+    pixel_setup<PDEG>(cam, op, px, py, in && px < cam.W && py < cam.H, oh, dh, Yh, valid);
+    float q[3] = {0.f, 0.f, 0.f}, hf = 0.f;
+    end[h] = 0;
+    if (valid) {
+      const size_t pix = (size_t)py * cam.W + px, plane = (size_t)cam.W * cam.H;
+      end[h] = view.n_used[pix];
+      q[0] = view.d_rgb[pix]; q[1] = view.d_rgb[plane + pix]; q[2] = view.d_rgb[2 * plane + pix];
+      hf = fmaf(q[0], view.rgb[pix], fmaf(q[1], view.rgb[plane + pix], q[2] * view.rgb[2 * plane + pix])) -
+           view.d_alpha[pix] * view.tfinal[pix];
+    }
+    pk[h] = end[h] > rg.x ? (uint32_t)px | ((uint32_t)py << 16) : kDead;
+    (h ? o.x.y : o.x.x) = oh.x; (h ? o.y.y : o.y.x) = oh.y; (h ? o.z.y : o.z.x) = oh.z;
+    (h ? d.x.y : d.x.x) = dh.x; (h ? d.y.y : d.y.x) = dh.y; (h ? d.z.y : d.z.x) = dh.z;
+#pragma unroll
+    for (int k = 0; k < PSH; ++k) (h ? Y[k].y : Y[k].x) = Yh[k];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) (h ? gr[c].y : gr[c].x) = q[c];
+    (h ? Hf.y : Hf.x) = hf;
+  }
+  // no pixel of this warp blends a particle at or after `stop`
+  const uint32_t stop = min(__reduce_max_sync(kFull, max(end[0], end[1])), rg.y);
+  if (stop <= rg.x) return;  // warp-uniform
+  warp_rays(pk, o, d, tile_is_8x8(op), lane, &S.rays);
+  if constexpr (!PP) {
+#pragma unroll
+    for (int k = 0; k < L::ROWS; ++k) {
+      uint2 hl = make_uint2(0u, 0u);
+      if (k < NSH) split_bf16x2(Y[k < NSH ? k : 0].x, Y[k < NSH ? k : 0].y, hl.x, hl.y);
+      S.A[k][pair_slot(k, lane)] = hl;
+    }
+  }
+  __syncwarp();
+
+  // Contracts the first `cols` columns of W with Y and adds the rows to the particles' SH
+  // gradients.  Columns past `cols` hold older values; they only feed their own, unread outputs.
   auto flush = [&](int cols) {
     __syncwarp();
     float acc[3][4];
 #pragma unroll
     for (int c = 0; c < 3; ++c) acc[c][0] = acc[c][1] = acc[c][2] = acc[c][3] = 0.f;
 #pragma unroll
-    for (int ks = 0; ks < 2; ++ks) {
-      const uint4 h4 = s_Af[(2 * ks) * 32 + lane], l4 = s_Af[(2 * ks + 1) * 32 + lane];
-      const uint32_t ahi[4] = {h4.x, h4.y, h4.z, h4.w}, alo[4] = {l4.x, l4.y, l4.z, l4.w};
+    for (int ks = 0; ks < 4; ++ks) {
+      const int l0 = pair_slot(g8, 8 * ks + t4), l1 = pair_slot(g8, 8 * ks + 4 + t4);
+      const uint2 z = make_uint2(0u, 0u);
+      const uint2 a0 = S.A[g8][l0], a2 = S.A[g8][l1];
+      const uint2 a1 = L::ROWS > 8 ? S.A[L::ROWS > 8 ? g8 + 8 : 0][l0] : z;
+      const uint2 a3 = L::ROWS > 8 ? S.A[L::ROWS > 8 ? g8 + 8 : 0][l1] : z;
+      const uint32_t ahi[4] = {a0.x, a1.x, a2.x, a3.x}, alo[4] = {a0.y, a1.y, a2.y, a3.y};
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const int row = c * kSlots + g8, c0 = 16 * ks + 2 * t4;
-        const float2 x0 = *reinterpret_cast<const float2 *>(s_W + wtile(row, c0));
-        const float2 x1 = *reinterpret_cast<const float2 *>(s_W + wtile(row, c0 + 8));
-        uint32_t bhi0, blo0, bhi1, blo1;
-        split_bf16x2(x0.x, x0.y, bhi0, blo0);
-        split_bf16x2(x1.x, x1.y, bhi1, blo1);
-        mma_bf16(acc[c], ahi, bhi0, bhi1);
-        mma_bf16(acc[c], ahi, blo0, blo1);
-        mma_bf16(acc[c], alo, bhi0, bhi1);
-      }
-    }
-    // acc[c][r]: basis g8 (+8 for r >= 2), column 2 t4 (+1 for odd r)
-    const int bA = __shfl_sync(0xffffffffu, slot_b, 2 * t4), bB = __shfl_sync(0xffffffffu, slot_b, 2 * t4 + 1);
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int k = g8 + (r >= 2 ? 8 : 0), col = 2 * t4 + (r & 1);
-      if (k < NSH && col < cols) {
-        float *dst = s_acc + (r & 1 ? bB : bA) * ACC + 16 + 3 * k;
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-          if (acc[c][r] != 0.f) atomicAdd(dst + c, acc[c][r]);
+        const uint2 b0 = S.W[c * kSlots + g8][l0], b1 = S.W[c * kSlots + g8][l1];
+        mma_bf16(acc[c], ahi, b0.x, b1.x);
+        mma_bf16(acc[c], ahi, b0.y, b1.y);
+        mma_bf16(acc[c], alo, b0.x, b1.x);
       }
     }
     __syncwarp();
+    // acc[c][r]: basis g8 (+8 for r >= 2), column 2 t4 (+1 for odd r)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int k = g8 + (r >= 2 ? 8 : 0), col = 2 * t4 + (r & 1);
+      if (k < NSH) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) S.out[col * L::OST + 3 * k + c] = acc[c][r];
+      }
+    }
+    __syncwarp();
+    add_rows<NC>(sc, S.out, L::OST, S.cidx, cols, lane);
+    __syncwarp();
   };
 
-  float T = 1.f, A0 = 0.f, A1 = 0.f, A2 = 0.f;  // running prefix of the composited colour
-  for (uint32_t start = rg.x; start < block_end; start += kBatch) {
-    const int nb = min((uint32_t)kBatch, block_end - start);
-    __syncthreads();
-    if (threadIdx.x < nb) s_idx[threadIdx.x] = vals[start + threadIdx.x];
-    for (int f = threadIdx.x; f < kBatch * ACC; f += blockDim.x) s_acc[f] = 0.f;
-    if (threadIdx.x < kBatch) s_any[threadIdx.x] = 0;
-    __syncthreads();
-    if (threadIdx.x < nb) {
-      uint32_t idx = s_idx[threadIdx.x];
-      stage_particle<RS>(sc, cam, op, rect[view.part_off + idx], idx, s_geo[threadIdx.x], &s_aux[threadIdx.x]);
-      if (PP) reinterpret_cast<float4 *>(s_sh)[threadIdx.x] = particle_colour<DEG, RS>(sc, cam, op, idx);
+  float2 T = bc(1.f), P = bc(0.f);  // transmittance, g . (running prefix of the composited colour)
+  int cols = 0;
+  uint32_t idx = list_index(vals, rg.x + lane, stop), idx1 = list_index(vals, rg.x + 32 + lane, stop);
+  short4 r = list_rect(rect, view.part_off, idx, rg.x + lane, stop);
+  for (uint32_t p0 = rg.x; p0 < stop;) {
+    const short4 r1 = list_rect(rect, view.part_off, idx1, p0 + 32 + lane, stop);
+    const uint32_t idx2 = list_index(vals, p0 + 64 + lane, stop);
+    bool near_ = rect_near(S.rays, r);
+    float4 g[4], aux;
+    if (near_) {
+      stage_particle<RS>(sc, cam, op, r, idx, g, &aux);
+      near_ = !block_misses<RS>(g, S.rays);
     }
-    if (!PP) stage_sh<NC>(sc, s_idx, nb, s_sh);
-    __syncthreads();
-    // particles of this batch any pixel of the warp can still blend (warp-uniform)
-    const int nw = (int)min((uint32_t)nb, warp_end > start ? warp_end - start : 0u);
-    int cols = 0;
-    for (int b = 0; b < nw; ++b) {
-      bool contrib = false;
-      float vv[3] = {0.f, 0.f, 0.f}, xx[3] = {0.f, 0.f, 0.f}, wc[3] = {0.f, 0.f, 0.f}, dsig = 0.f;
-      float3 og, dg;
-      float dd, a;
-      if (start + b < my_end && eval_response<RS, GEN>(s_geo[b], px, py, o, d, og, dg, dd, a, op)) {
-        contrib = true;
-        float al = fminf(a, op.alpha_max);
-        float r0, r1, r2;
-        if (PP) {
-          const float4 cr = reinterpret_cast<const float4 *>(s_sh)[b];
-          r0 = cr.x; r1 = cr.y; r2 = cr.z;
-        } else {
-          sh_colour<NSH>(s_sh + b * NC, Y, r0, r1, r2);
-        }
-        float c0 = fmaxf(r0, 0.f), c1 = fmaxf(r1, 0.f), c2 = fmaxf(r2, 0.f);
-        float w = al * T;
-        A0 = fmaf(c0, w, A0);
-        A1 = fmaf(c1, w, A1);
-        A2 = fmaf(c2, w, A2);
-        const float inv = __fdividef(1.f, 1.f - al);  // 1 - al >= 1 - alpha_max > 0
-        // dL/dalpha = sum_c g_c (c T - S_c / (1 - alpha)) + g_A T_final / (1 - alpha)
-        float dal = g0 * fmaf(-(Cf0 - A0), inv, c0 * T) + g1 * fmaf(-(Cf1 - A1), inv, c1 * T) +
-                    g2 * fmaf(-(Cf2 - A2), inv, c2 * T) + gAT * inv;
-        wc[0] = r0 > 0.f ? g0 * w : 0.f;
-        wc[1] = r1 > 0.f ? g1 * w : 0.f;
-        wc[2] = r2 > 0.f ? g2 * w : 0.f;
-        T = T * (1.f - al);
-        float da = a > op.alpha_max ? 0.f : dal;
-        float sigma = s_geo[b][3].x;
-        dsig = da * __fdividef(a, sigma);
-        float dw2 = dresponse<GEN>(op, a, og, dg, dd) * da;
-        float tau = -__fdividef(dot3(og, dg), dd);
-        float3 pp = make_float3(fmaf(tau, dg.x, og.x), fmaf(tau, dg.y, og.y), fmaf(tau, dg.z, og.z));
-        vv[0] = 2.f * dw2 * pp.x;
-        vv[1] = 2.f * dw2 * pp.y;
-        vv[2] = 2.f * dw2 * pp.z;
-        float4 ax = s_aux[b];
-        if (RS) {
-          xx[0] = fmaf(tau, d.x, o.x - ax.x);
-          xx[1] = fmaf(tau, d.y, o.y - ax.y);
-          xx[2] = fmaf(tau, d.z, o.z - ax.z);
-        } else {
-          xx[0] = fmaf(tau, d.x, ax.x);
-          xx[1] = fmaf(tau, d.y, ax.y);
-          xx[2] = fmaf(tau, d.z, ax.z);
-        }
-      }
-      if (!__any_sync(0xffffffffu, contrib)) continue;
-      if (!PP) {
-        // SH weights into the next free column of W (row = channel x column, entry = pixel)
+    const unsigned m = __ballot_sync(kFull, near_);
+    const int b0 = __popc(m & ((1u << lane) - 1u)), n = min(__popc(m), kRoundB);
+    // survivors past the round's room are left to the next one
+    const unsigned over = __ballot_sync(kFull, near_ && b0 >= kRoundB);
+    if (near_ && b0 < kRoundB) {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) s_W[wtile(c * kSlots + cols, lane)] = wc[c];
-        if (lane == cols) slot_b = b;
+      for (int q = 0; q < 4; ++q) S.geo[b0][q] = g[q];
+      aux.w = __uint_as_float(p0 + lane);
+      S.geo[b0][4] = aux;
+      S.idx[b0] = idx;
+      if (PP) {
+        reinterpret_cast<float4 *>(S.col)[b0] = particle_colour<DEG, RS>(sc, cam, op, idx);
+        S.dc[PP ? b0 : 0][0] = S.dc[PP ? b0 : 0][1] = S.dc[PP ? b0 : 0][2] = 0.f;
       }
+    }
+    __syncwarp();
+    if (!PP) stage_sh_warp<NC>(sc, S.idx, n, S.col, lane);
+    for (int b = 0; b < n; ++b) {  // warp-uniform
+      const float4 g3 = S.geo[b][3], ax = S.geo[b][4];
+      const uint32_t q0 = __float_as_uint(g3.z), q1 = __float_as_uint(g3.w), pos = __float_as_uint(ax.w);
+      bool h0 = in_rect(pk[0], q0, q1) && pos < end[0], h1 = in_rect(pk[1], q0, q1) && pos < end[1];
+      float2 wc[3] = {bc(0.f), bc(0.f), bc(0.f)};
       float v[16];
-      v[0] = vv[0]; v[1] = vv[1]; v[2] = vv[2];
 #pragma unroll
-      for (int r = 0; r < 3; ++r)
+      for (int k = 0; k < 16; ++k) v[k] = 0.f;
+      if (h0 || h1) {
+        const PairEval e = eval_pair<RS>(S.geo[b][0], S.geo[b][1], S.geo[b][2], o, d);
+        h0 = h0 && e.cc.x <= g3.y * e.dd.x;
+        h1 = h1 && e.cc.y <= g3.y * e.dd.y;
+        if (h0 || h1) {
+          // a pixel that the particle does not reach has alpha 0 and takes part in no sum
+          const float2 a = make_float2(h0 ? response<GEN>(g3.x, e.cc.x, e.dd.x, op) : 0.f,
+                                       h1 ? response<GEN>(g3.x, e.cc.y, e.dd.y, op) : 0.f);
+          const float2 al = make_float2(fminf(a.x, op.alpha_max), fminf(a.y, op.alpha_max));
+          float2 c0, c1, c2;
+          if (PP) {
+            const float4 cr = reinterpret_cast<const float4 *>(S.col)[b];
+            c0 = bc(cr.x); c1 = bc(cr.y); c2 = bc(cr.z);
+          } else {
+            sh_colour2<NSH>(S.col + b * NC, Y, c0, c1, c2);
+          }
+          c0 = make_float2(h0 ? fmaxf(c0.x, 0.f) : 0.f, h1 ? fmaxf(c0.y, 0.f) : 0.f);
+          c1 = make_float2(h0 ? fmaxf(c1.x, 0.f) : 0.f, h1 ? fmaxf(c1.y, 0.f) : 0.f);
+          c2 = make_float2(h0 ? fmaxf(c2.x, 0.f) : 0.f, h1 ? fmaxf(c2.y, 0.f) : 0.f);
+          const float2 w = mul2(al, T);
+          const float2 gc = fma2(gr[0], c0, fma2(gr[1], c1, mul2(gr[2], c2)));
+          P = fma2(gc, w, P);
+          const float2 om = make_float2(1.f - al.x, 1.f - al.y);  // >= 1 - alpha_max > 0
+          const float2 inv = make_float2(__fdividef(1.f, om.x), __fdividef(1.f, om.y));
+          // dL/dalpha = sum_c g_c (c T - S_c / (1 - alpha)) + g_A T_final / (1 - alpha) with the
+          // colour still to come S = C - prefix: g . S - g_A T_final = Hf - P
+          const float2 dal = fma2(gc, T, mul2(add2(P, neg2(Hf)), inv));
+          wc[0] = make_float2(c0.x > 0.f ? gr[0].x * w.x : 0.f, c0.y > 0.f ? gr[0].y * w.y : 0.f);
+          wc[1] = make_float2(c1.x > 0.f ? gr[1].x * w.x : 0.f, c1.y > 0.f ? gr[1].y * w.y : 0.f);
+          wc[2] = make_float2(c2.x > 0.f ? gr[2].x * w.x : 0.f, c2.y > 0.f ? gr[2].y * w.y : 0.f);
+          T = mul2(T, om);
+          const float2 da = make_float2(!h0 || a.x > op.alpha_max ? 0.f : dal.x,
+                                        !h1 || a.y > op.alpha_max ? 0.f : dal.y);
+          v[12] = fmaf(da.x, __fdividef(a.x, g3.x), da.y * __fdividef(a.y, g3.x));
+          // 2 dL/domega^2
+          float2 dw = make_float2(-a.x * da.x, -a.y * da.y);
+          if (GEN) dw = make_float2(2.f * dresponse_w2(op, a.x, h0 ? __fdividef(e.cc.x, e.dd.x) : 0.f) * da.x,
+                                    2.f * dresponse_w2(op, a.y, h1 ? __fdividef(e.cc.y, e.dd.y) : 0.f) * da.y);
+          const float2 od = dot3x2(e.og, e.dg);
+          const float2 tau = make_float2(h0 ? -__fdividef(od.x, e.dd.x) : 0.f, h1 ? -__fdividef(od.y, e.dd.y) : 0.f);
+          const float2 vv[3] = {mul2(dw, fma2(tau, e.dg.x, e.og.x)), mul2(dw, fma2(tau, e.dg.y, e.og.y)),
+                                mul2(dw, fma2(tau, e.dg.z, e.og.z))};
+          f3x2 x;
+          if (RS) {
+            x.x = add2(o.x, bc(-ax.x));
+            x.y = add2(o.y, bc(-ax.y));
+            x.z = add2(o.z, bc(-ax.z));
+          } else {
+            x.x = bc(ax.x);
+            x.y = bc(ax.y);
+            x.z = bc(ax.z);
+          }
+          const float2 xx[3] = {fma2(tau, d.x, x.x), fma2(tau, d.y, x.y), fma2(tau, d.z, x.z)};
 #pragma unroll
-        for (int c = 0; c < 3; ++c) v[3 + 3 * r + c] = vv[r] * xx[c];
-      v[12] = dsig;
-      v[13] = PP ? wc[0] : 0.f;
-      v[14] = PP ? wc[1] : 0.f;
-      v[15] = PP ? wc[2] : 0.f;
+          for (int q = 0; q < 3; ++q) {
+            v[q] = vv[q].x + vv[q].y;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) v[3 + 3 * q + c] = fmaf(vv[q].x, xx[c].x, vv[q].y * xx[c].y);
+          }
+        }
+      }
+      if (!__any_sync(kFull, h0 || h1)) continue;
+      const uint32_t pi = S.idx[b];
+      if (PP) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) v[13 + c] = wc[c].x + wc[c].y;
+      } else {
+        // SH weights into the next free column of W
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          uint2 hl;
+          split_bf16x2(wc[c].x, wc[c].y, hl.x, hl.y);
+          S.W[PP ? 0 : c * kSlots + cols][pair_slot(cols, lane)] = hl;
+        }
+        if (lane == 0) S.cidx[cols] = pi;
+      }
       warp_reduce_scatter16(v, lane);
       const int vi = (lane >> 1) & 15;
-      if (!(lane & 1) && vi < (PP ? 16 : 13)) atomicAdd(&s_acc[b * ACC + vi], v[0]);
-      if (lane == 0) s_any[b] = 1;
+      if (!(lane & 1)) {
+        if (vi < 13) atomicAdd(&sc.gacc[(size_t)pi * 16 + vi], v[0]);
+        else if (PP) S.dc[PP ? b : 0][vi - 13] = v[0];
+      }
       if (!PP && ++cols == kSlots) {
         flush(kSlots);
         cols = 0;
       }
     }
-    if (!PP && cols > 0) flush(cols);
-    __syncthreads();
-    for (int f = threadIdx.x; f < nb * ACC; f += blockDim.x) {
-      int b = f / ACC, j = f - b * ACC;
-      if (!s_any[b]) continue;
-      uint32_t idx = s_idx[b];
-      float v = s_acc[f];
-      if (j < 13) atomicAdd(&sc.gacc[(size_t)idx * 16 + j], v);
-      else if (!PP && j >= 16 && j < 16 + NC) atomicAdd(&sc.d_sh[(size_t)idx * NC + (j - 16)], v);
-    }
-    if (PP) {
-      // dL/dc of this tile's pixels -> dL/dbeta_k,ch = dL/dc_ch Y_k(dir) and the mean's gradient
+    if constexpr (PP) {
+      // dL/dc of this warp's pixels -> dL/dbeta_k,ch = dL/dc_ch Y_k(dir) and the mean's gradient
       // through dir = (mu - c) / |mu - c|: (I - dir dir^T) / |mu - c| sum_ch dL/dc_ch grad c_ch
-      for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-        if (!s_any[b]) continue;
-        const float g0c = s_acc[b * ACC + 13], g1c = s_acc[b * ACC + 14], g2c = s_acc[b * ACC + 15];
-        if (g0c == 0.f && g1c == 0.f && g2c == 0.f) continue;
-        const uint32_t idx = s_idx[b];
-        const float3 mu = make_float3(sc.means[3 * idx], sc.means[3 * idx + 1], sc.means[3 * idx + 2]);
+      __syncwarp();
+      const bool row = lane < n;
+      const float g0c = row ? S.dc[row ? lane : 0][0] : 0.f, g1c = row ? S.dc[row ? lane : 0][1] : 0.f,
+                  g2c = row ? S.dc[row ? lane : 0][2] : 0.f;
+      const bool some = !(g0c == 0.f && g1c == 0.f && g2c == 0.f);
+      const unsigned rows = __ballot_sync(kFull, some);
+      if (some) {
+        const uint32_t pi = S.idx[lane];
+        const int b = __popc(rows & ((1u << lane) - 1u));
+        const float3 mu = make_float3(sc.means[3 * pi], sc.means[3 * pi + 1], sc.means[3 * pi + 2]);
         float il;
         const float3 dir = particle_dir<RS>(cam, op, mu, il);
         float Yp[NSH], a[NSH];
         sh_basis<DEG>(dir.x, dir.y, dir.z, Yp);
-        const float *beta = sc.sh + (size_t)idx * NC;
-        float *dsh = sc.d_sh + (size_t)idx * NC;
+        const float *beta = sc.sh + (size_t)pi * NC;
+        float *dsh = S.out + b * L::OST;
+        S.cidx[b] = pi;
 #pragma unroll
         for (int k = 0; k < NSH; ++k) {
           a[k] = fmaf(g0c, beta[3 * k], fmaf(g1c, beta[3 * k + 1], g2c * beta[3 * k + 2]));
-          if (g0c != 0.f) atomicAdd(&dsh[3 * k], g0c * Yp[k]);
-          if (g1c != 0.f) atomicAdd(&dsh[3 * k + 1], g1c * Yp[k]);
-          if (g2c != 0.f) atomicAdd(&dsh[3 * k + 2], g2c * Yp[k]);
+          dsh[3 * k] = g0c * Yp[k];
+          dsh[3 * k + 1] = g1c * Yp[k];
+          dsh[3 * k + 2] = g2c * Yp[k];
         }
         const float3 G = sh_poly_grad<DEG>(dir.x, dir.y, dir.z, a);
         const float gd = dot3(G, dir);
-        atomicAdd(&sc.gacc[(size_t)idx * 16 + 13], (G.x - gd * dir.x) * il);
-        atomicAdd(&sc.gacc[(size_t)idx * 16 + 14], (G.y - gd * dir.y) * il);
-        atomicAdd(&sc.gacc[(size_t)idx * 16 + 15], (G.z - gd * dir.z) * il);
+        atomicAdd(&sc.gacc[(size_t)pi * 16 + 13], (G.x - gd * dir.x) * il);
+        atomicAdd(&sc.gacc[(size_t)pi * 16 + 14], (G.y - gd * dir.y) * il);
+        atomicAdd(&sc.gacc[(size_t)pi * 16 + 15], (G.z - gd * dir.z) * il);
       }
+      __syncwarp();
+      add_rows<NC>(sc, S.out, L::OST, S.cidx, __popc(rows), lane);
+    }
+    __syncwarp();  // the survivors are read before the next round's are staged
+    if (over) {
+      p0 += __ffs(over) - 1;
+      idx = list_index(vals, p0 + lane, stop);
+      idx1 = list_index(vals, p0 + 32 + lane, stop);
+      r = list_rect(rect, view.part_off, idx, p0 + lane, stop);
+    } else {
+      p0 += 32;
+      idx = idx1;
+      idx1 = idx2;
+      r = r1;
     }
   }
+  if (!PP && cols > 0) flush(cols);
 }
 
 // One warp per tile: work = list entries the backward replays (up to one past the last
@@ -432,22 +495,14 @@ __global__ void k_finalize(const __grid_constant__ BatchDesc bd, int total) {
   }
 }
 
-template <int DEG, bool RS, bool SMALL, bool PP, bool GEN>
+template <int DEG, bool RS, bool PP, bool GEN>
 void bwd_launch_k(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, const uint32_t *vals,
                   const uint32_t *ranges, const TileSched &ts, cudaStream_t s) {
-  const int blocks = bd.total_tiles, threads = op.tile_w * op.tile_h;
-  const size_t smem = BwdSmem<DEG, PP>::bytes(threads / 32);
-  cudaFuncSetAttribute(k_composite_bwd<DEG, RS, SMALL, PP, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)smem);
-  k_composite_bwd<DEG, RS, SMALL, PP, GEN><<<blocks, threads, smem, s>>>(
+  const int warps = block_warps(op);
+  const size_t smem = sizeof(BwdWarp<DEG, PP>) * (size_t)warps;
+  cudaFuncSetAttribute(k_composite_bwd<DEG, RS, PP, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_composite_bwd<DEG, RS, PP, GEN><<<bd.total_tiles * tile_blocks(op), 32 * warps, smem, s>>>(
       bd, op, reinterpret_cast<const short4 *>(rect), vals, reinterpret_cast<const uint2 *>(ranges), ts);
-}
-
-template <int DEG, bool RS, bool PP, bool GEN>
-void bwd_launch_pp(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, const uint32_t *vals,
-                   const uint32_t *ranges, const TileSched &ts, cudaStream_t s) {
-  if (op.tile_w * op.tile_h <= 256) bwd_launch_k<DEG, RS, true, PP, GEN>(bd, op, rect, vals, ranges, ts, s);
-  else bwd_launch_k<DEG, RS, false, PP, GEN>(bd, op, rect, vals, ranges, ts, s);
 }
 
 // Degree 0 colours do not depend on the direction: both colour modes run the per-pixel kernel.
@@ -457,16 +512,16 @@ template <int DEG, bool RS>
 void bwd_launch(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, const uint32_t *vals,
                 const uint32_t *ranges, const TileSched &ts, cudaStream_t s) {
   if (op.kernel_degree != 2) {
-    bwd_launch_pp<DEG, RS, false, true>(bd, op, rect, vals, ranges, ts, s);
+    bwd_launch_k<DEG, RS, false, true>(bd, op, rect, vals, ranges, ts, s);
     return;
   }
   if constexpr (DEG > 0) {
     if (op.colour_mode == UT_COLOUR_PER_PARTICLE) {
-      bwd_launch_pp<DEG, RS, true, false>(bd, op, rect, vals, ranges, ts, s);
+      bwd_launch_k<DEG, RS, true, false>(bd, op, rect, vals, ranges, ts, s);
       return;
     }
   }
-  bwd_launch_pp<DEG, RS, false, false>(bd, op, rect, vals, ranges, ts, s);
+  bwd_launch_k<DEG, RS, false, false>(bd, op, rect, vals, ranges, ts, s);
 }
 
 }  // namespace

@@ -4,11 +4,11 @@
 // (supplementary Sec. A), SH colour (per pixel or per particle), pixel setup, and the tile
 // schedule both passes use (a counting sort of the tiles by their expected walk, longest first).
 //
-// One thread block per image tile (global tile ids over all views of the batch), one thread
-// per pixel.  The tile's depth-sorted particle list is consumed in batches: the block gathers
-// each batch's parameters once, activates them (M = S^-1 R^T, sigma, the alpha_min test
-// threshold, packed rect) into shared memory together with their colour data, and every pixel
-// then walks the batch from shared memory.
+// The tile-order forward and backward walk a tile with independent warps (composite_warp.cuh).
+// The k-buffer kernels use one block per tile and one thread per pixel: the tile's depth-sorted
+// list is consumed in batches whose parameters the block activates (M = S^-1 R^T, sigma, the
+// alpha_min test threshold, packed rect) into shared memory together with their colour data, and
+// every pixel walks the batch from there.
 //
 // Template RS selects the general ray-origin path (per-pixel origin, needed when any view
 // has a rolling shutter); without it the origin is the camera centre of the view.
@@ -21,8 +21,6 @@
 namespace ut3d {
 namespace {
 
-constexpr int kBatch = 64;    // particles staged per block step (backward)
-constexpr int kBatchF = 128;  // particles staged per block step (forward)
 constexpr int kBatchK = 64;   // particles staged per block step (k-buffer): two blocks of 256 fit an SM
 constexpr int kOrderBuckets = 1024;  // log buckets of the backward's tile schedule
 
@@ -171,12 +169,8 @@ __device__ __forceinline__ bool eval_response(const float4 *g, int px, int py, f
   return true;
 }
 
-// d rho / d omega^2 times sigma, from a = sigma rho at the response's omega^2.
-template <bool GEN>
-__device__ __forceinline__ float dresponse(const DevOpts &op, float a, float3 og, float3 dg, float dd) {
-  if (!GEN) return -0.5f * a;
-  const float3 c = cross3(og, dg);
-  const float w2 = __fdividef(fmaf(c.x, c.x, fmaf(c.y, c.y, c.z * c.z)), dd);
+// d rho / d omega^2 times sigma for the degree-n kernel, from a = sigma rho at omega^2 = w2.
+__device__ __forceinline__ float dresponse_w2(const DevOpts &op, float a, float w2) {
   return -op.kernel_lambda * 0.5f * (float)op.kernel_degree * pow_half(w2, op.kernel_degree - 2) * a;
 }
 

@@ -72,6 +72,7 @@ struct DevScene {
   float *d_means, *d_log_scales, *d_quats, *d_logits, *d_sh;
   int grad_off;                 // flattened offset of this scene in finalize's range
   int sh_vec;                   // sh is 16-byte aligned and (deg+1)^2 * 3 is a multiple of 4
+  int dsh_vec;                  // the same of d_sh
 };
 
 struct BatchDesc {
