@@ -135,7 +135,6 @@ __global__ void __launch_bounds__(32 * kBlockWarps, 3) k_composite_bwd(const __g
   constexpr int NSH = L::NSH;
   constexpr int NC = L::NC;
   constexpr int PDEG = PP ? 0 : DEG;  // per-pixel SH basis only when colours are per pixel
-  constexpr int PSH = (PDEG + 1) * (PDEG + 1);
   extern __shared__ __align__(16) unsigned char smem[];
 
   // tiles in the order k_tile_order gave them (most list entries to replay first)
@@ -155,35 +154,25 @@ __global__ void __launch_bounds__(32 * kBlockWarps, 3) k_composite_bwd(const __g
   const int x0 = (lt % view.tiles_x) * op.tile_w, y0 = (lt / view.tiles_x) * op.tile_h;
   const uint2 rg = ranges[tile];
 
-  f3x2 o, d;
-  float2 Y[PSH];
+  PixelPair<PDEG> q;
+  pixel_pair<PDEG>(cam, op, x0, y0, warp, lane, q);
+  const f3x2 o = q.o, d = q.d;
   uint32_t pk[2], end[2];  // the pixels with something to replay (kDead: none), and where each stops
   float2 gr[3], Hf;  // upstream g = dL/drgb, and g . (composited colour) - dL/dalpha T_final
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    int lx, ly;
-    const bool in = tile_pixel2(op, warp, lane, h, lx, ly);
-    const int px = x0 + lx, py = y0 + ly;
-    float3 oh, dh;
-    float Yh[PSH];
-    bool valid;
-    pixel_setup<PDEG>(cam, op, px, py, in && px < cam.W && py < cam.H, oh, dh, Yh, valid);
-    float q[3] = {0.f, 0.f, 0.f}, hf = 0.f;
+    float u[3] = {0.f, 0.f, 0.f}, hf = 0.f;
     end[h] = 0;
-    if (valid) {
-      const size_t pix = (size_t)py * cam.W + px, plane = (size_t)cam.W * cam.H;
+    if (q.valid[h]) {
+      const size_t pix = (size_t)q.py[h] * cam.W + q.px[h], plane = (size_t)cam.W * cam.H;
       end[h] = view.n_used[pix];
-      q[0] = view.d_rgb[pix]; q[1] = view.d_rgb[plane + pix]; q[2] = view.d_rgb[2 * plane + pix];
-      hf = fmaf(q[0], view.rgb[pix], fmaf(q[1], view.rgb[plane + pix], q[2] * view.rgb[2 * plane + pix])) -
+      u[0] = view.d_rgb[pix]; u[1] = view.d_rgb[plane + pix]; u[2] = view.d_rgb[2 * plane + pix];
+      hf = fmaf(u[0], view.rgb[pix], fmaf(u[1], view.rgb[plane + pix], u[2] * view.rgb[2 * plane + pix])) -
            view.d_alpha[pix] * view.tfinal[pix];
     }
-    pk[h] = end[h] > rg.x ? (uint32_t)px | ((uint32_t)py << 16) : kDead;
-    (h ? o.x.y : o.x.x) = oh.x; (h ? o.y.y : o.y.x) = oh.y; (h ? o.z.y : o.z.x) = oh.z;
-    (h ? d.x.y : d.x.x) = dh.x; (h ? d.y.y : d.y.x) = dh.y; (h ? d.z.y : d.z.x) = dh.z;
+    pk[h] = end[h] > rg.x ? (uint32_t)q.px[h] | ((uint32_t)q.py[h] << 16) : kDead;
 #pragma unroll
-    for (int k = 0; k < PSH; ++k) (h ? Y[k].y : Y[k].x) = Yh[k];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) (h ? gr[c].y : gr[c].x) = q[c];
+    for (int c = 0; c < 3; ++c) (h ? gr[c].y : gr[c].x) = u[c];
     (h ? Hf.y : Hf.x) = hf;
   }
   // no pixel of this warp blends a particle at or after `stop`
@@ -194,7 +183,7 @@ __global__ void __launch_bounds__(32 * kBlockWarps, 3) k_composite_bwd(const __g
 #pragma unroll
     for (int k = 0; k < L::ROWS; ++k) {
       uint2 hl = make_uint2(0u, 0u);
-      if (k < NSH) split_bf16x2(Y[k < NSH ? k : 0].x, Y[k < NSH ? k : 0].y, hl.x, hl.y);
+      if (k < NSH) split_bf16x2(q.Y[k < NSH ? k : 0].x, q.Y[k < NSH ? k : 0].y, hl.x, hl.y);
       S.A[k][pair_slot(k, lane)] = hl;
     }
   }
@@ -290,7 +279,7 @@ __global__ void __launch_bounds__(32 * kBlockWarps, 3) k_composite_bwd(const __g
             const float4 cr = reinterpret_cast<const float4 *>(S.col)[b];
             c0 = bc(cr.x); c1 = bc(cr.y); c2 = bc(cr.z);
           } else {
-            sh_colour2<NSH>(S.col + b * NC, Y, c0, c1, c2);
+            sh_colour2<NSH>(S.col + b * NC, q.Y, c0, c1, c2);
           }
           c0 = make_float2(h0 ? fmaxf(c0.x, 0.f) : 0.f, h1 ? fmaxf(c0.y, 0.f) : 0.f);
           c1 = make_float2(h0 ? fmaxf(c1.x, 0.f) : 0.f, h1 ? fmaxf(c1.y, 0.f) : 0.f);

@@ -18,6 +18,18 @@ struct __align__(16) FwdWarp {
   uint32_t idx[kRoundF], pos[kRoundF];  // particle, list position
 };
 
+// A pixel's outputs (alpha is 0 where it has no ray: its T stays 1).
+__device__ __forceinline__ void store_pixel(const DevView &view, const DevCam &cam, int px, int py, float c0, float c1,
+                                            float c2, float T, uint32_t last) {
+  const size_t pix = (size_t)py * cam.W + px, plane = (size_t)cam.W * cam.H;
+  view.rgb[pix] = c0;
+  view.rgb[plane + pix] = c1;
+  view.rgb[2 * plane + pix] = c2;
+  view.alpha[pix] = 1.f - T;
+  if (view.tfinal) view.tfinal[pix] = T;
+  if (view.n_used) view.n_used[pix] = last;
+}
+
 // Resident blocks of 128 threads per SM that the kernel is compiled for.  Bound by issue and by the
 // latency of a chunk's loads, so more warps pay until the pixels' state spills.  Measured per call:
 // degree 3 on the 1M rolling-shutter 1080p view 1172 us a frame at 4 blocks (128 registers),
@@ -42,15 +54,13 @@ __global__ void __launch_bounds__(32 * kBlockWarps, fwd_blocks(DEG, RS, PP)) k_c
   constexpr int NSH = (DEG + 1) * (DEG + 1);
   constexpr int NC = NSH * 3;
   constexpr int PDEG = PP ? 0 : DEG;        // per-pixel SH basis only when colours are per pixel
-  constexpr int PSH = (PDEG + 1) * (PDEG + 1);
   constexpr int NST = PP ? 4 : NC;          // staged colour floats per particle
   extern __shared__ __align__(16) unsigned char smem[];
 
   // tiles in the order k_tile_order gave them (longest predicted walk first); every tile is
   // in the order, so every pixel is written
   const uint32_t rank = blockIdx.x / (uint32_t)tile_blocks(op);
-  if (rank >= *ts.n_work) return;
-  const int tile = (int)ts.order[rank];
+  const int tile = (int)(ts.order ? ts.order[rank] : rank);
   UT_DBG_CHECK(tile < bd.total_tiles, UT_DBG_TILE_ID, tile, bd.total_tiles, 2);
   const DevView &view = bd.v[view_of_tile(bd, tile)];
   const DevScene &sc = bd.s[view.scene];
@@ -62,34 +72,31 @@ __global__ void __launch_bounds__(32 * kBlockWarps, fwd_blocks(DEG, RS, PP)) k_c
   const int lt = tile - view.tile_off;
   const int x0 = (lt % view.tiles_x) * op.tile_w, y0 = (lt / view.tiles_x) * op.tile_h;
 
-  f3x2 o, d;
-  float2 Y[PSH];
+  const uint2 rg = ranges[tile];
+  if (rg.x >= rg.y) {  // nothing to composite: no rays needed
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      int lx, ly;
+      if (tile_pixel2(op, warp, lane, h, lx, ly) && x0 + lx < cam.W && y0 + ly < cam.H)
+        store_pixel(view, cam, x0 + lx, y0 + ly, 0.f, 0.f, 0.f, 1.f, 0u);
+    }
+    return;
+  }
+  // entries of this chunk of 32 and of the next one (their rectangles are loaded a chunk ahead)
+  uint32_t idx = list_index(vals, rg.x + lane, rg.y), idx1 = list_index(vals, rg.x + 32 + lane, rg.y);
+  short4 r = list_rect(rect, view.part_off, idx, rg.x + lane, rg.y);
+  PixelPair<PDEG> q;
+  pixel_pair<PDEG>(cam, op, x0, y0, warp, lane, q);
+  const f3x2 o = q.o, d = q.d;
   uint32_t pk[2];  // the pixels still walking, kDead once stopped
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    int lx, ly;
-    const bool in = tile_pixel2(op, warp, lane, h, lx, ly);
-    const int px = x0 + lx, py = y0 + ly;
-    float3 oh, dh;
-    float Yh[PSH];
-    bool valid;
-    pixel_setup<PDEG>(cam, op, px, py, in && px < cam.W && py < cam.H, oh, dh, Yh, valid);
-    pk[h] = valid ? (uint32_t)px | ((uint32_t)py << 16) : kDead;
-    (h ? o.x.y : o.x.x) = oh.x; (h ? o.y.y : o.y.x) = oh.y; (h ? o.z.y : o.z.x) = oh.z;
-    (h ? d.x.y : d.x.x) = dh.x; (h ? d.y.y : d.y.x) = dh.y; (h ? d.z.y : d.z.x) = dh.z;
-#pragma unroll
-    for (int k = 0; k < PSH; ++k) (h ? Y[k].y : Y[k].x) = Yh[k];
-  }
+  for (int h = 0; h < 2; ++h) pk[h] = q.valid[h] ? (uint32_t)q.px[h] | ((uint32_t)q.py[h] << 16) : kDead;
   warp_rays(pk, o, d, tile_is_8x8(op), lane, &S.rays);
   __syncwarp();
 
   float T[2] = {1.f, 1.f}, C[2][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
   uint32_t last[2] = {0u, 0u};
   unsigned long long n_eval = 0, n_blend = 0;
-  const uint2 rg = ranges[tile];
-  // entries of this chunk of 32 and of the next one (their rectangles are loaded a chunk ahead)
-  uint32_t idx = list_index(vals, rg.x + lane, rg.y), idx1 = list_index(vals, rg.x + 32 + lane, rg.y);
-  short4 r = list_rect(rect, view.part_off, idx, rg.x + lane, rg.y);
   for (uint32_t p0 = rg.x; p0 < rg.y; p0 += 32) {
     if (__all_sync(kFull, pk[0] == kDead && pk[1] == kDead)) break;
     const short4 r1 = list_rect(rect, view.part_off, idx1, p0 + 32 + lane, rg.y);
@@ -140,7 +147,7 @@ __global__ void __launch_bounds__(32 * kBlockWarps, fwd_blocks(DEG, RS, PP)) k_c
         const float4 c = reinterpret_cast<const float4 *>(S.col)[b];
         c0 = bc(c.x); c1 = bc(c.y); c2 = bc(c.z);
       } else {
-        sh_colour2<NSH>(S.col + b * NC, Y, c0, c1, c2);
+        sh_colour2<NSH>(S.col + b * NC, q.Y, c0, c1, c2);
       }
       if (h0) {
         const float w = al0 * T[0];
@@ -167,18 +174,10 @@ __global__ void __launch_bounds__(32 * kBlockWarps, fwd_blocks(DEG, RS, PP)) k_c
     r = r1;
   }
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  for (int h = 0; h < 2; ++h) {  // (the coordinates are recomputed, not kept through the walk)
     int lx, ly;
-    const bool in = tile_pixel2(op, warp, lane, h, lx, ly);
-    const int px = x0 + lx, py = y0 + ly;
-    if (!in || px >= cam.W || py >= cam.H) continue;
-    const size_t pix = (size_t)py * cam.W + px, plane = (size_t)cam.W * cam.H;
-    view.rgb[pix] = C[h][0];
-    view.rgb[plane + pix] = C[h][1];
-    view.rgb[2 * plane + pix] = C[h][2];
-    view.alpha[pix] = 1.f - T[h];  // 0 where the pixel has no ray: T stays 1
-    if (view.tfinal) view.tfinal[pix] = T[h];
-    if (view.n_used) view.n_used[pix] = last[h];
+    if (tile_pixel2(op, warp, lane, h, lx, ly) && x0 + lx < cam.W && y0 + ly < cam.H)
+      store_pixel(view, cam, x0 + lx, y0 + ly, C[h][0], C[h][1], C[h][2], T[h], last[h]);
   }
   if (STATS) {
     for (int s = 16; s >= 1; s >>= 1) {
@@ -213,8 +212,7 @@ __global__ void __launch_bounds__(512, 1) k_composite_fwd_kbuffer(const __grid_c
   __shared__ uint32_t s_idx[kBatchK];
   extern __shared__ float s_kb[];  // [6][k][threads]: tau, alpha, r, g, b, list position of each hit
 
-  if (blockIdx.x >= *ts.n_work) return;
-  const int tile = (int)ts.order[blockIdx.x];
+  const int tile = (int)(ts.order ? ts.order[blockIdx.x] : blockIdx.x);
   UT_DBG_CHECK(tile < bd.total_tiles, UT_DBG_TILE_ID, tile, bd.total_tiles, 2);
   const DevView &view = bd.v[view_of_tile(bd, tile)];
   const DevScene &sc = bd.s[view.scene];
@@ -429,13 +427,21 @@ ut_status launch_composite_fwd(const BatchDesc &bd, const DevOpts &op, const int
                                const uint32_t *ranges, unsigned long long *stats, void *sched, cudaStream_t s) {
   if (op.kbuffer > 0 && stats) return UT_ERR_UNSUPPORTED;
   if (bd.total_tiles == 0) return UT_OK;
-  const TileSched ts = carve_tile_sched(sched, bd.total_tiles);
-  if (cudaMemsetAsync(ts.hist, 0, sizeof(uint32_t) * (2 * kOrderBuckets + 1), s) != cudaSuccess) return UT_ERR_CUDA;
-  k_fwd_predict<<<(bd.total_tiles + 7) / 8, 256, 0, s>>>(bd, op, reinterpret_cast<const short4 *>(rect), vals,
-                                                         reinterpret_cast<const uint2 *>(ranges), ts);
-  const int ob = (bd.total_tiles + kOrderBuckets - 1) / kOrderBuckets, cap = device_sm_count();
-  k_tile_order<<<ob < cap ? ob : cap, kOrderBuckets, 0, s>>>(bd.total_tiles, ts);
-  count_launches(2);
+  TileSched ts = carve_tile_sched(sched, bd.total_tiles);
+  // when every block is resident at once (4 a SM at least, 1 for the k-buffer) the order does not
+  // matter: the prediction's launches would only delay the frame
+  const int sms = device_sm_count();
+  const long long blocks = (long long)bd.total_tiles * (op.kbuffer > 0 ? 1 : tile_blocks(op));
+  if (blocks <= (op.kbuffer > 0 ? 1 : 4) * sms) {
+    ts.order = nullptr;
+  } else {
+    if (cudaMemsetAsync(ts.hist, 0, sizeof(uint32_t) * (2 * kOrderBuckets + 1), s) != cudaSuccess) return UT_ERR_CUDA;
+    k_fwd_predict<<<(bd.total_tiles + 7) / 8, 256, 0, s>>>(bd, op, reinterpret_cast<const short4 *>(rect), vals,
+                                                           reinterpret_cast<const uint2 *>(ranges), ts);
+    const int ob = (bd.total_tiles + kOrderBuckets - 1) / kOrderBuckets;
+    k_tile_order<<<ob < sms ? ob : sms, kOrderBuckets, 0, s>>>(bd.total_tiles, ts);
+    count_launches(2);
+  }
   const bool rs = any_rs(bd);
 #define UT3D_FWD(D)                                                     \
   (rs ? fwd_launch<D, true>(bd, op, rect, vals, ranges, stats, ts, s) \

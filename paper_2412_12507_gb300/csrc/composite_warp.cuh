@@ -160,6 +160,52 @@ __device__ __forceinline__ bool tile_pixel2(const DevOpts &op, int warp, int lan
 // A pixel as x | y << 16 (both below 2^15), or kDead: never inside a rectangle.
 constexpr uint32_t kDead = 0x80008000u;
 
+// The pair's pixels, rays and SH basis: px, py, whether each lies in its tile and image, whether it
+// has a ray (pixel_setup's results, both pixels in step).
+template <int DEG>
+struct PixelPair {
+  int px[2], py[2];
+  bool in[2], valid[2];
+  f3x2 o, d;
+  float2 Y[(DEG + 1) * (DEG + 1)];
+};
+
+template <int DEG>
+__device__ __forceinline__ void pixel_pair(const DevCam &cam, const DevOpts &op, int x0, int y0, int warp, int lane,
+                                           PixelPair<DEG> &q) {
+  constexpr int NSH = (DEG + 1) * (DEG + 1);
+  PixelPlane p[2];
+  float rd[2], x[2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    int lx, ly;
+    q.in[h] = tile_pixel2(op, warp, lane, h, lx, ly);
+    q.px[h] = x0 + lx;
+    q.py[h] = y0 + ly;
+    q.in[h] = q.in[h] && q.px[h] < cam.W && q.py[h] < cam.H;
+    p[h] = pixel_plane(cam, q.px[h], q.py[h]);
+    rd[h] = p[h].rd;
+    q.valid[h] = q.in[h] && imaged(cam, p[h]);
+  }
+  undistort<2>(cam, rd, q.valid, op.newton_iters, x);
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    float3 o = make_float3(0.f, 0.f, 1.f), d = o;
+    float Y[NSH];
+#pragma unroll
+    for (int k = 0; k < NSH; ++k) Y[k] = 0.f;
+    if (q.valid[h]) {
+      ray_of(cam, q.py[h], p[h], x[h], o, d);
+      const float in = rsqrtf(dot3(d, d));
+      sh_basis<DEG>(d.x * in, d.y * in, d.z * in, Y);
+    }
+    (h ? q.o.x.y : q.o.x.x) = o.x; (h ? q.o.y.y : q.o.y.x) = o.y; (h ? q.o.z.y : q.o.z.x) = o.z;
+    (h ? q.d.x.y : q.d.x.x) = d.x; (h ? q.d.y.y : q.d.y.x) = d.y; (h ? q.d.z.y : q.d.z.x) = d.z;
+#pragma unroll
+    for (int k = 0; k < NSH; ++k) (h ? q.Y[k].y : q.Y[k].x) = Y[k];
+  }
+}
+
 __device__ __forceinline__ bool in_rect(uint32_t p, uint32_t r0, uint32_t r1) {
   return __vmins2(__vmaxs2(p, r0), r1) == p;  // per 16-bit half: clamping to [r0, r1] keeps p
 }

@@ -382,52 +382,84 @@ __device__ __forceinline__ bool project_world(const DevCam &c, int rs_iters, flo
               : project_world_t<UT_CAM_FISHEYE, false>(c, rs_iters, y, uv, t_out);
 }
 
-// World ray of pixel (px, py) (integer indices; the ray goes through the pixel centre).
-// Returns false for a fisheye pixel outside the imaged disc.
-__device__ __forceinline__ bool pixel_ray(const DevCam &c, int px, int py, int newton_iters, float3 &o, float3 &d) {
-  float mx = (px + 0.5f - c.cx) * c.ifx;
-  float my = (py + 0.5f - c.cy) * c.ify;
+// Normalised image coordinates of a pixel centre, and their radius (0 for a pinhole).
+struct PixelPlane {
+  float mx, my, rd;
+};
+
+__device__ __forceinline__ PixelPlane pixel_plane(const DevCam &c, int px, int py) {
+  PixelPlane p;
+  p.mx = (px + 0.5f - c.cx) * c.ifx;
+  p.my = (py + 0.5f - c.cy) * c.ify;
+  p.rd = c.model == UT_CAM_PINHOLE ? 0.f : sqrtf(fmaf(p.mx, p.mx, p.my * p.my));
+  return p;
+}
+
+// The undistorted radius (radial pinhole) or angle (fisheye) of P image radii: a safeguarded Newton
+// iteration for r_d(r) = rd or theta_d(theta) = rd on the increasing branch [0, theta_max].  The P
+// iterations run in step (a radius that has converged keeps its value), so their latencies
+// overlap; each takes exactly the steps it would take alone.  Radii with live[] false are left 0.
+// In FP32 the iteration often ends in two neighbouring values that step to each other; since both
+// then bound the bracket they do so for ever, and the value that the last of newton_iters steps
+// would leave follows from the number of steps left.
+template <int P>
+__device__ __forceinline__ void undistort(const DevCam &c, const float (&rd)[P], const bool (&live)[P],
+                                          int newton_iters, float (&x)[P]) {
+  const bool radial = c.model == UT_CAM_PINHOLE_RADIAL;
+  float lo[P], hi[P], prev[P];  // prev: the iterate that a Newton step led to x from
+  bool run[P];
+#pragma unroll
+  for (int h = 0; h < P; ++h) {
+    lo[h] = x[h] = hi[h] = 0.f;
+    prev[h] = -1.f;  // no iterate is negative
+    run[h] = live[h];
+    if (!run[h] || c.model == UT_CAM_PINHOLE) continue;
+    hi[h] = radial ? fminf(c.theta_max, fmaxf(2.f * rd[h], 1.f)) : c.theta_max;
+    if (radial)
+      for (int it = 0; it < 40 && isinf(c.theta_max) && rd[h] > hi[h] * radial_scale(c, hi[h] * hi[h]); ++it)
+        hi[h] *= 2.f;
+    x[h] = fminf(rd[h], hi[h]);
+  }
+  if (c.model == UT_CAM_PINHOLE) return;
+  for (int it = 0; it < newton_iters; ++it) {
+    bool any = false;
+#pragma unroll
+    for (int h = 0; h < P; ++h) {
+      const float v = x[h], v2 = v * v;
+      const float f = radial ? fmaf(v, radial_scale(c, v2), -rd[h]) : theta_d_poly(c, v) - rd[h];
+      float nv = v - f / (radial ? radial_prime(c, v2) : theta_d_prime(c, v));
+      if (run[h]) {
+        run[h] = f != 0.f;
+        if (run[h]) {
+          if (f > 0.f) hi[h] = v; else lo[h] = v;
+          const bool newton = nv >= lo[h] && nv <= hi[h];
+          if (!newton) nv = 0.5f * (lo[h] + hi[h]);  // Newton left the bracket: bisect
+          const bool cycle = newton && nv == prev[h];
+          run[h] = nv != v && !cycle;
+          x[h] = cycle && ((newton_iters - 1 - it) & 1) ? v : nv;
+          prev[h] = newton ? v : -1.f;
+        }
+      }
+      any |= run[h];
+    }
+    if (!any) break;
+  }
+}
+
+// World ray of pixel (px, py) (integer indices; the ray goes through the pixel centre) from its
+// undistorted radius or angle x.
+__device__ __forceinline__ void ray_of(const DevCam &c, int py, const PixelPlane &p, float x, float3 &o, float3 &d) {
   float3 dc;
   if (c.model == UT_CAM_PINHOLE) {
-    dc = make_float3(mx, my, 1.f);
+    dc = make_float3(p.mx, p.my, 1.f);
   } else if (c.model == UT_CAM_PINHOLE_RADIAL) {
-    float rd = sqrtf(fmaf(mx, mx, my * my));
-    if (!(rd <= c.rd_max)) return false;
-    // safeguarded Newton for r_d(r) = rd on the increasing branch [0, r_max]
-    float lo = 0.f, hi = fminf(c.theta_max, fmaxf(2.f * rd, 1.f));
-    for (int it = 0; it < 40 && isinf(c.theta_max) && rd > hi * radial_scale(c, hi * hi); ++it) hi *= 2.f;
-    float r = fminf(rd, hi);
-    for (int it = 0; it < newton_iters; ++it) {
-      float f = fmaf(r, radial_scale(c, r * r), -rd);
-      if (f == 0.f) break;
-      if (f > 0.f) hi = r; else lo = r;
-      float nr = r - f / radial_prime(c, r * r);
-      if (!(nr >= lo && nr <= hi)) nr = 0.5f * (lo + hi);  // Newton left the bracket: bisect
-      if (nr == r) break;
-      r = nr;
-    }
-    dc = rd > 0.f ? make_float3(mx * (r / rd), my * (r / rd), 1.f) : make_float3(0.f, 0.f, 1.f);
+    dc = p.rd > 0.f ? make_float3(p.mx * (x / p.rd), p.my * (x / p.rd), 1.f) : make_float3(0.f, 0.f, 1.f);
   } else {
-    float rd = sqrtf(fmaf(mx, mx, my * my));
-    if (!(rd <= c.rd_max)) return false;
-    // safeguarded Newton for theta_d(theta) = rd on the increasing branch [0, theta_max]
-    float lo = 0.f, hi = c.theta_max;
-    float th = fminf(rd, c.theta_max);
-    for (int it = 0; it < newton_iters; ++it) {
-      float f = theta_d_poly(c, th) - rd;
-      if (f == 0.f) break;
-      if (f > 0.f) hi = th; else lo = th;
-      float fp = theta_d_prime(c, th);
-      float nt = th - f / fp;
-      if (!(nt >= lo && nt <= hi)) nt = 0.5f * (lo + hi);  // Newton left the bracket: bisect
-      if (nt == th) break;
-      th = nt;
-    }
     float s, co;
-    sincosf(th, &s, &co);
-    if (rd > 0.f) {
-      float k = s / rd;
-      dc = make_float3(k * mx, k * my, co);
+    sincosf(x, &s, &co);
+    if (p.rd > 0.f) {
+      float k = s / p.rd;
+      dc = make_float3(k * p.mx, k * p.my, co);
     } else {
       dc = make_float3(0.f, 0.f, 1.f);
     }
@@ -445,6 +477,21 @@ __device__ __forceinline__ bool pixel_ray(const DevCam &c, int px, int py, int n
     o = mat3_tmul(c.R0, make_float3(-Tt.x, -Tt.y, -Tt.z));
     d = mat3_tmul(c.R0, dc);
   }
+}
+
+// Whether a pixel has a ray: false outside the imaged disc of a fisheye or radial camera.
+__device__ __forceinline__ bool imaged(const DevCam &c, const PixelPlane &p) {
+  return c.model == UT_CAM_PINHOLE || p.rd <= c.rd_max;
+}
+
+__device__ __forceinline__ bool pixel_ray(const DevCam &c, int px, int py, int newton_iters, float3 &o, float3 &d) {
+  const PixelPlane p = pixel_plane(c, px, py);
+  if (!imaged(c, p)) return false;
+  const float rd[1] = {p.rd};
+  const bool live[1] = {true};
+  float x[1];
+  undistort<1>(c, rd, live, newton_iters, x);
+  ray_of(c, py, p, x[0], o, d);
   return true;
 }
 
