@@ -27,16 +27,6 @@ constexpr unsigned kFull = 0xffffffffu;
 
 // ---------------------------------------------------------------- packed pairs (one value per pixel)
 
-__device__ __forceinline__ float2 bc(float x) { return make_float2(x, x); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
-
-struct f3x2 {
-  float2 x, y, z;
-};
-
 __device__ __forceinline__ float2 dot3x2(const f3x2 &a, const f3x2 &b) {
   return fma2(a.x, b.x, fma2(a.y, b.y, mul2(a.z, b.z)));
 }

@@ -27,6 +27,20 @@ __device__ __forceinline__ bool proj_world(const DevCam &c, int rs_iters, float3
   else return project_world_t<CAM / 2, (CAM & 1) != 0>(c, rs_iters, y, uv, t);
 }
 
+// Two points at once (packed arithmetic, the same results).
+template <int CAM>
+__device__ __forceinline__ bool proj_world2(const DevCam &c, int rs_iters, const f3x2 &y, float2 &u, float2 &v) {
+  if constexpr (CAM >= 0) return project_world2<CAM / 2, (CAM & 1) != 0>(c, rs_iters, y, u, v);
+  if (c.model == UT_CAM_PINHOLE)
+    return c.rs ? project_world2<UT_CAM_PINHOLE, true>(c, rs_iters, y, u, v)
+                : project_world2<UT_CAM_PINHOLE, false>(c, rs_iters, y, u, v);
+  if (c.model == UT_CAM_PINHOLE_RADIAL)
+    return c.rs ? project_world2<UT_CAM_PINHOLE_RADIAL, true>(c, rs_iters, y, u, v)
+                : project_world2<UT_CAM_PINHOLE_RADIAL, false>(c, rs_iters, y, u, v);
+  return c.rs ? project_world2<UT_CAM_FISHEYE, true>(c, rs_iters, y, u, v)
+              : project_world2<UT_CAM_FISHEYE, false>(c, rs_iters, y, u, v);
+}
+
 template <int CAM>
 __device__ __forceinline__ float3 point_at(const DevCam &c, float3 y, float t) {
   if constexpr (CAM < 0) return cam_point_at(c, y, t);
@@ -104,7 +118,7 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_project(const __grid_constan
     }
   } else {
     // sigma points in start-pose camera rotation: y_0 = R0 mu, y = y_0 +- gamma s_k R0 R[:,k].
-    // The six off-centre points go through one (not unrolled) loop, each projection taken
+    // The six off-centre points go through one (not unrolled) loop, two at a time, each projection taken
     // relative to the centre's v_0 (d_j = v_j - v_0), which keeps the moments free of
     // cancellation: eq. 2d_conic_1 gives v_mu = v_0 + wi sum d_j (the mean weights sum to one)
     // and eq. 2d_conic_2 gives Sigma' = wi sum d_j d_j^T + (W - 2) dm dm^T with dm = wi sum d_j
@@ -119,19 +133,26 @@ __global__ void __launch_bounds__(kWarps * 32, 4) k_project(const __grid_constan
     }
     float sx = 0.f, sy = 0.f, pxx = 0.f, pxy = 0.f, pyy = 0.f;
 #pragma unroll 1
-    for (int j = 0; j < 6; ++j) {
-      const int k = j < 3 ? j : j - 3;
-      const float3 c3 = k == 0 ? col[0] : (k == 1 ? col[1] : col[2]);  // selects, no local memory
-      const float3 dy = j < 3 ? c3 : make_float3(-c3.x, -c3.y, -c3.z);
-      float2 v;
-      float tt;
-      ok = ok & proj_world<CAM>(cam, op.rs_iters, make_float3(y0.x + dy.x, y0.y + dy.y, y0.z + dy.z), v, tt);
-      const float dx = v.x - v0.x, dz = v.y - v0.y;
-      sx += dx;
-      sy += dz;
-      pxx = fmaf(dx, dx, pxx);
-      pxy = fmaf(dx, dz, pxy);
-      pyy = fmaf(dz, dz, pyy);
+    for (int j = 0; j < 3; ++j) {  // points (+0, +1), (+2, -0), (-1, -2), summed in that order
+      const float3 a = j == 0 ? col[0] : (j == 1 ? col[2] : make_float3(-col[1].x, -col[1].y, -col[1].z));
+      const float3 e = j == 0 ? col[1] : (j == 1 ? make_float3(-col[0].x, -col[0].y, -col[0].z)
+                                                 : make_float3(-col[2].x, -col[2].y, -col[2].z));
+      f3x2 y;
+      y.x = add2(bc(y0.x), make_float2(a.x, e.x));
+      y.y = add2(bc(y0.y), make_float2(a.y, e.y));
+      y.z = add2(bc(y0.z), make_float2(a.z, e.z));
+      float2 u, v;
+      ok = ok & proj_world2<CAM>(cam, op.rs_iters, y, u, v);
+      const float2 dx = sub2(u, bc(v0.x)), dz = sub2(v, bc(v0.y));
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float x = h ? dx.y : dx.x, z = h ? dz.y : dz.x;
+        sx += x;
+        sy += z;
+        pxx = fmaf(x, x, pxx);
+        pxy = fmaf(x, z, pxy);
+        pyy = fmaf(z, z, pyy);
+      }
     }
     const float dmx = w.wi * sx, dmy = w.wi * sy;
     const float c = w.wc0 + 6.f * w.wi - 2.f;

@@ -134,6 +134,25 @@ __device__ __forceinline__ int scene_of_grad(const BatchDesc &b, int g) {
   return lo;
 }
 
+// ---------------------------------------------------------------- packed FP32 pairs
+//
+// One fma.rn.f32x2 instruction does two FMAs, each rounded like fmaf: kernels bound by instruction
+// issue handle two pixels or two sigma points at a time.
+__device__ __forceinline__ float2 bc(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+struct f3x2 {
+  float2 x, y, z;
+};
+
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return add2(a, neg2(b)); }
+__device__ __forceinline__ float2 sel2(bool x, bool y, float2 a, float2 b) {
+  return make_float2(x ? a.x : b.x, y ? a.y : b.y);
+}
+
 __device__ __forceinline__ float3 mat3_mul(const float *R, float3 v) {
   return make_float3(fmaf(R[0], v.x, fmaf(R[1], v.y, R[2] * v.z)), fmaf(R[3], v.x, fmaf(R[4], v.y, R[5] * v.z)),
                      fmaf(R[6], v.x, fmaf(R[7], v.y, R[8] * v.z)));
@@ -444,6 +463,128 @@ __device__ __forceinline__ void undistort(const DevCam &c, const float (&rd)[P],
     }
     if (!any) break;
   }
+}
+
+// ---------------------------------------------------------------- two points at a time
+//
+// The pair forms of sincos_pi, rotate_axis(_fast), cam_project(_fast)_t and project_world_t: the same
+// operations in the same order for each point, with the FMAs packed.
+__device__ __forceinline__ void sincos_pi2(float2 th, float2 &s, float2 &c) {
+  const float2 k = make_float2(rintf(th.x * 0.63661977236758134f), rintf(th.y * 0.63661977236758134f));
+  float2 r = fma2(neg2(k), bc(1.5707963705062866f), th);
+  r = fma2(neg2(k), bc(-4.371139000186243e-08f), r);
+  const float2 r2 = mul2(r, r);
+  const float2 sr = fma2(mul2(r, r2), fma2(r2, fma2(r2, bc(-1.9496e-4f), bc(8.33198e-3f)), bc(-0.16666651f)), r);
+  const float2 cr = fma2(mul2(r2, r2), fma2(r2, fma2(r2, bc(2.44385385e-05f), bc(-1.38873683e-03f)), bc(4.16666469e-02f)),
+                         fma2(bc(-0.5f), r2, bc(1.f)));
+  const int q0 = ((int)k.x) & 3, q1 = ((int)k.y) & 3;
+  const float2 ss = sel2(q0 & 1, q1 & 1, cr, sr), cc = sel2(q0 & 1, q1 & 1, sr, cr);
+  s = sel2(q0 & 2, q1 & 2, neg2(ss), ss);
+  c = sel2(q0 == 1 || q0 == 2, q1 == 1 || q1 == 2, neg2(cc), cc);
+}
+
+template <bool FAST>
+__device__ __forceinline__ f3x2 rotate_axis2(const float *a, const f3x2 &y, float2 th) {
+  float2 s, c;
+  if (FAST) {
+    __sincosf(th.x, &s.x, &c.x);
+    __sincosf(th.y, &s.y, &c.y);
+  } else {
+    sincos_pi2(th, s, c);
+  }
+  const float2 ad = fma2(bc(a[2]), y.z, fma2(bc(a[0]), y.x, mul2(bc(a[1]), y.y)));
+  const f3x2 v = {fma2(bc(a[1]), y.z, neg2(mul2(bc(a[2]), y.y))), fma2(bc(a[2]), y.x, neg2(mul2(bc(a[0]), y.z))),
+                  fma2(bc(a[0]), y.y, neg2(mul2(bc(a[1]), y.x)))};
+  const float2 oc = mul2(sub2(bc(1.f), c), ad);
+  return {fma2(y.x, c, fma2(v.x, s, mul2(bc(a[0]), oc))), fma2(y.y, c, fma2(v.y, s, mul2(bc(a[1]), oc))),
+          fma2(y.z, c, fma2(v.z, s, mul2(bc(a[2]), oc)))};
+}
+
+__device__ __forceinline__ float2 theta_d_poly2(const DevCam &c, float2 th) {
+  const float2 t2 = mul2(th, th);
+  return mul2(th, fma2(t2, fma2(t2, fma2(t2, fma2(t2, bc(c.k4), bc(c.k3)), bc(c.k2)), bc(c.k1)), bc(1.f)));
+}
+
+__device__ __forceinline__ float2 radial_scale2(const DevCam &c, float2 r2) {
+  return fma2(r2, fma2(r2, fma2(r2, bc(c.k3), bc(c.k2)), bc(c.k1)), bc(1.f));
+}
+
+__device__ __forceinline__ float2 atan2_pos_fast2(float2 y, float2 x) {
+  const float2 ax = make_float2(fabsf(x.x), fabsf(x.y));
+  const float2 mx = make_float2(fmaxf(y.x, ax.x), fmaxf(y.y, ax.y)), mn = make_float2(fminf(y.x, ax.x), fminf(y.y, ax.y));
+  const float2 a = make_float2(mx.x > 0.f ? __fdividef(mn.x, mx.x) : 0.f, mx.y > 0.f ? __fdividef(mn.y, mx.y) : 0.f);
+  const float2 a2 = mul2(a, a);
+  float2 p = bc(-0.004054596647620201f);
+  p = fma2(p, a2, bc(0.021863065659999847f));
+  p = fma2(p, a2, bc(-0.05591248348355293f));
+  p = fma2(p, a2, bc(0.09642209112644196f));
+  p = fma2(p, a2, bc(-0.13908633589744568f));
+  p = fma2(p, a2, bc(0.19946566224098206f));
+  p = fma2(p, a2, bc(-0.33329862356185913f));
+  p = fma2(p, a2, bc(0.9999993443489075f));
+  float2 r = mul2(p, a);
+  r = sel2(y.x > ax.x, y.y > ax.y, sub2(bc(1.5707963267948966f), r), r);
+  return sel2(x.x < 0.f, x.y < 0.f, sub2(bc(3.141592653589793f), r), r);
+}
+
+// g of a pair of camera-space points; FAST: cam_project_fast_t's operations, else cam_project_t's.
+// Returns false when either is not imaged.
+template <int MODEL, bool FAST>
+__device__ __forceinline__ bool cam_project2(const DevCam &c, const f3x2 &p, float2 &u, float2 &v) {
+  if constexpr (MODEL == UT_CAM_FISHEYE) {
+    const float2 r2 = fma2(p.x, p.x, mul2(p.y, p.y));
+    float2 rq = make_float2(rsqrtf(r2.x), rsqrtf(r2.y));
+    if (!FAST) rq = mul2(rq, fma2(mul2(bc(-0.5f), r2), mul2(rq, rq), bc(1.5f)));
+    const bool ax0 = !(r2.x > 0.f), ax1 = !(r2.y > 0.f);
+    const float2 rho = sel2(ax0, ax1, bc(0.f), mul2(r2, rq));
+    const float2 th = FAST ? atan2_pos_fast2(rho, p.z) : make_float2(atan2f(rho.x, p.z.x), atan2f(rho.y, p.z.y));
+    float2 s = mul2(theta_d_poly2(c, th), rq);
+    if (ax0) s.x = FAST ? __fdividef(1.f, p.z.x) : 1.f / p.z.x;
+    if (ax1) s.y = FAST ? __fdividef(1.f, p.z.y) : 1.f / p.z.y;
+    u = fma2(mul2(bc(c.fx), s), p.x, bc(c.cx));
+    v = fma2(mul2(bc(c.fy), s), p.y, bc(c.cy));
+    const float2 d2 = fma2(p.z, p.z, r2);
+    const float n2 = c.near_plane * c.near_plane;
+    return d2.x > n2 && d2.y > n2 && th.x <= c.theta_max && th.y <= c.theta_max;
+  } else {
+    const float2 iz = FAST ? make_float2(__fdividef(1.f, p.z.x), __fdividef(1.f, p.z.y))
+                           : make_float2(1.f / p.z.x, 1.f / p.z.y);
+    bool ok = p.z.x > c.near_plane && p.z.y > c.near_plane;
+    if constexpr (MODEL == UT_CAM_PINHOLE_RADIAL) {
+      const float2 xn = mul2(p.x, iz), yn = mul2(p.y, iz);
+      const float2 r2 = fma2(xn, xn, mul2(yn, yn));
+      const float2 sd = radial_scale2(c, r2);
+      u = fma2(mul2(bc(c.fx), xn), sd, bc(c.cx));
+      v = fma2(mul2(bc(c.fy), yn), sd, bc(c.cy));
+      if (FAST) ok = ok && r2.x <= c.theta_max * c.theta_max && r2.y <= c.theta_max * c.theta_max;
+      else ok = ok && sqrtf(r2.x) <= c.theta_max && sqrtf(r2.y) <= c.theta_max;
+    } else {
+      u = fma2(mul2(bc(c.fx), p.x), iz, bc(c.cx));
+      v = fma2(mul2(bc(c.fy), p.y), iz, bc(c.cy));
+    }
+    return ok;
+  }
+}
+
+// project_world_t of two points (y = R0 x each).
+template <int MODEL, bool RS>
+__device__ __forceinline__ bool project_world2(const DevCam &c, int rs_iters, const f3x2 &y, float2 &u, float2 &v) {
+  bool ok = true;
+  float2 t = bc(0.f);
+  auto at = [&](const f3x2 &r) -> f3x2 {
+    return {add2(r.x, fma2(t, bc(c.dT[0]), bc(c.T0[0]))), add2(r.y, fma2(t, bc(c.dT[1]), bc(c.T0[1]))),
+            add2(r.z, fma2(t, bc(c.dT[2]), bc(c.T0[2])))};
+  };
+  if (RS) {
+    t = bc(0.5f);
+    for (int it = 0; it < rs_iters; ++it) {
+      ok &= cam_project2<MODEL, true>(c, at(rotate_axis2<true>(c.ax, y, mul2(t, bc(c.phi)))), u, v);
+      const float2 w = mul2(add2(v, bc(-0.5f)), bc(c.inv_hm1));
+      t = make_float2(fminf(fmaxf(w.x, 0.f), 1.f), fminf(fmaxf(w.y, 0.f), 1.f));
+    }
+  }
+  ok &= cam_project2<MODEL, false>(c, at(RS ? rotate_axis2<false>(c.ax, y, mul2(t, bc(c.phi))) : y), u, v);
+  return ok;
 }
 
 // World ray of pixel (px, py) (integer indices; the ray goes through the pixel centre) from its
