@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(32 * kBlockWarps, 3) k_composite_bwd(const __g
   // no pixel of this warp blends a particle at or after `stop`
   const uint32_t stop = min(__reduce_max_sync(kFull, max(end[0], end[1])), rg.y);
   if (stop <= rg.x) return;  // warp-uniform
-  warp_rays(pk, o, d, tile_is_8x8(op), lane, &S.rays);
+  warp_rays(pk, o, d, tile_is_8x8(op) ? 8 : 0, lane, &S.rays);
   if constexpr (!PP) {
 #pragma unroll
     for (int k = 0; k < L::ROWS; ++k) {
@@ -540,7 +540,7 @@ ut_status launch_composite_bwd(const BatchDesc &bd, const DevOpts &op, const int
     total = sc.grad_off + sc.n > total ? sc.grad_off + sc.n : total;
   }
   if (op.kbuffer > 0) {  // "Ours (sorted)": its own replay of the per-ray k-buffer
-    const ut_status st = launch_composite_bwd_kbuffer(bd, op, rect, vals, ranges, s);
+    const ut_status st = launch_composite_bwd_kbuffer(bd, op, rect, vals, ranges, sched, s);
     if (st != UT_OK) return st;
   } else if (bd.total_tiles > 0) {
     const TileSched ts = carve_tile_sched(sched, bd.total_tiles);

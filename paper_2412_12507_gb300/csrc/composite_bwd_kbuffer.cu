@@ -22,7 +22,7 @@
 // blend the same particle at nearly the same time, and shared-memory atomics on one address
 // serialise, while the L2's reductions absorb them).
 // Selection by tau_max is piecewise constant and carries no gradient.
-#include "composite_common.cuh"
+#include "composite_warp.cuh"
 
 namespace ut3d {
 namespace {
@@ -65,16 +65,16 @@ template <int DEG, bool RS>
 __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_constant__ BatchDesc bd, DevOpts op,
                                                                const short4 *__restrict__ rect,
                                                                const uint32_t *__restrict__ vals,
-                                                               const uint2 *__restrict__ ranges) {
+                                                               const uint2 *__restrict__ ranges, TileSched ts) {
   constexpr int NSH = (DEG + 1) * (DEG + 1);
   constexpr int NC = NSH * 3;
   __shared__ float4 s_geo[kBatchKB][4];
   __shared__ float4 s_aux[kBatchKB];
   __shared__ __align__(16) float s_sh[kBatchKB * NC];
   __shared__ uint32_t s_idx[kBatchKB];
-  extern __shared__ float s_kb[];  // [6][k][threads]: tau, alpha, r, g, b, list position
+  extern __shared__ __align__(16) float s_kb[];  // [6][k][threads]: tau, alpha, r, g, b, list position; [warps] rays
 
-  const int tile = blockIdx.x;
+  const int tile = (int)(ts.order ? ts.order[blockIdx.x] : blockIdx.x);
   const DevView &view = bd.v[view_of_tile(bd, tile)];
   const DevScene &sc = bd.s[view.scene];
   const DevCam &cam = view.cam;
@@ -184,6 +184,8 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
 
   // adds this step's blend events to the particles' accumulators; every lane of the warp calls it
   const int lane = threadIdx.x & 31;
+  WarpRays &rays = reinterpret_cast<WarpRays *>(s_kb + 6 * K * nt)[threadIdx.x >> 5];
+  warp_rays1(op, px, py, o, d, valid, lane, &rays);
   auto emit = [&]() {
     const unsigned act = __ballot_sync(0xffffffffu, has_ev);
     if (!act) return;
@@ -252,8 +254,13 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
     sb = start;
     snb = nb;
     if (__all_sync(0xffffffffu, done)) continue;
-    // every lane of the warp walks every staged particle (the emit steps are warp-wide)
-    for (int b = 0; b < nb; ++b) {
+    // every lane of the warp walks every particle that can reach its pixels (the emit steps are
+    // warp-wide)
+    for (int c0 = 0; c0 < nb; c0 += 32) {
+    unsigned m = near_mask<RS>(s_geo, c0, nb, rays, lane);
+    while (m) {
+      const int b = c0 + __ffs(m) - 1;
+      m &= m - 1;
       float3 og, dg;
       float dd, a;
       bool leave = false;
@@ -288,6 +295,8 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
       emit();
       if (__all_sync(0xffffffffu, done)) break;
     }
+    if (__all_sync(0xffffffffu, done)) break;
+    }
   }
   // end of the list: the remaining hits in ascending (tau_max, arrival), the warp in step
   while (__any_sync(0xffffffffu, !done && nbuf > 0)) {
@@ -305,9 +314,9 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
 
 template <int DEG, bool RS>
 ut_status launch_k(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, const uint32_t *vals,
-                   const uint32_t *ranges, cudaStream_t s) {
+                   const uint32_t *ranges, const TileSched &ts, cudaStream_t s) {
   const int threads = op.tile_w * op.tile_h;
-  const size_t smem = sizeof(float) * 6 * (size_t)op.kbuffer * threads;
+  const size_t smem = sizeof(float) * 6 * (size_t)op.kbuffer * threads + sizeof(WarpRays) * (threads / 32);
   constexpr size_t kStatic = sizeof(float4) * kBatchKB * 5 + sizeof(float) * kBatchKB * 3 * (DEG + 1) * (DEG + 1) +
                              sizeof(uint32_t) * kBatchKB;
   if (smem + kStatic > 227 * 1024) return UT_ERR_UNSUPPORTED;  // the buffer does not fit one block
@@ -317,7 +326,7 @@ ut_status launch_k(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, 
                            cudaSharedmemCarveoutMaxShared) != cudaSuccess)
     return UT_ERR_CUDA;
   k_composite_bwd_kbuffer<DEG, RS><<<bd.total_tiles, threads, smem, s>>>(
-      bd, op, reinterpret_cast<const short4 *>(rect), vals, reinterpret_cast<const uint2 *>(ranges));
+      bd, op, reinterpret_cast<const short4 *>(rect), vals, reinterpret_cast<const uint2 *>(ranges), ts);
   count_launches(1);
   return UT_OK;
 }
@@ -326,7 +335,7 @@ ut_status launch_k(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, 
 
 // The k-buffer backward over every tile of the batch (accumulators cleared by the caller).
 ut_status launch_composite_bwd_kbuffer(const BatchDesc &bd, const DevOpts &op, const int16_t *rect,
-                                       const uint32_t *vals, const uint32_t *ranges, cudaStream_t s) {
+                                       const uint32_t *vals, const uint32_t *ranges, void *sched, cudaStream_t s) {
   if (bd.total_tiles == 0) return UT_OK;
   for (int k = 0; k < bd.ns; ++k) {
     const DevScene &sc = bd.s[k];
@@ -336,12 +345,17 @@ ut_status launch_composite_bwd_kbuffer(const BatchDesc &bd, const DevOpts &op, c
     k_kb_records<<<g < cap ? g : cap, 256, 0, s>>>(sc);
     count_launches(1);
   }
+  // tiles by predicted walk, longest first (n_used, which orders the tile-order backward, is not
+  // kept by the k-buffer); pointless when every tile is resident at once
+  TileSched ts = carve_tile_sched(sched, bd.total_tiles);
+  if (bd.total_tiles <= device_sm_count()) ts.order = nullptr;
+  else if (ut_status st = launch_walk_order(bd, op, rect, vals, ranges, sched, s); st != UT_OK) return st;
   const bool rs = any_rs(bd);
   switch (bd.s[0].deg) {
-    case 0: return rs ? launch_k<0, true>(bd, op, rect, vals, ranges, s) : launch_k<0, false>(bd, op, rect, vals, ranges, s);
-    case 1: return rs ? launch_k<1, true>(bd, op, rect, vals, ranges, s) : launch_k<1, false>(bd, op, rect, vals, ranges, s);
-    case 2: return rs ? launch_k<2, true>(bd, op, rect, vals, ranges, s) : launch_k<2, false>(bd, op, rect, vals, ranges, s);
-    default: return rs ? launch_k<3, true>(bd, op, rect, vals, ranges, s) : launch_k<3, false>(bd, op, rect, vals, ranges, s);
+    case 0: return rs ? launch_k<0, true>(bd, op, rect, vals, ranges, ts, s) : launch_k<0, false>(bd, op, rect, vals, ranges, ts, s);
+    case 1: return rs ? launch_k<1, true>(bd, op, rect, vals, ranges, ts, s) : launch_k<1, false>(bd, op, rect, vals, ranges, ts, s);
+    case 2: return rs ? launch_k<2, true>(bd, op, rect, vals, ranges, ts, s) : launch_k<2, false>(bd, op, rect, vals, ranges, ts, s);
+    default: return rs ? launch_k<3, true>(bd, op, rect, vals, ranges, ts, s) : launch_k<3, false>(bd, op, rect, vals, ranges, ts, s);
   }
 }
 

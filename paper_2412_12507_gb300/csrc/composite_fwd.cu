@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(32 * kBlockWarps, fwd_blocks(DEG, RS, PP)) k_c
   uint32_t pk[2];  // the pixels still walking, kDead once stopped
 #pragma unroll
   for (int h = 0; h < 2; ++h) pk[h] = q.valid[h] ? (uint32_t)q.px[h] | ((uint32_t)q.py[h] << 16) : kDead;
-  warp_rays(pk, o, d, tile_is_8x8(op), lane, &S.rays);
+  warp_rays(pk, o, d, tile_is_8x8(op) ? 8 : 0, lane, &S.rays);
   __syncwarp();
 
   float T[2] = {1.f, 1.f}, C[2][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(512, 1) k_composite_fwd_kbuffer(const __grid_c
   __shared__ float4 s_geo[kBatchK][4];
   __shared__ __align__(16) float s_sh[kBatchK * NC];
   __shared__ uint32_t s_idx[kBatchK];
-  extern __shared__ float s_kb[];  // [6][k][threads]: tau, alpha, r, g, b, list position of each hit
+  extern __shared__ __align__(16) float s_kb[];  // [6][k][threads]: tau, alpha, r, g, b, list position; [warps] rays
 
   const int tile = (int)(ts.order ? ts.order[blockIdx.x] : blockIdx.x);
   UT_DBG_CHECK(tile < bd.total_tiles, UT_DBG_TILE_ID, tile, bd.total_tiles, 2);
@@ -232,6 +232,10 @@ __global__ void __launch_bounds__(512, 1) k_composite_fwd_kbuffer(const __grid_c
   float Y[NSH];
   bool valid;
   pixel_setup<DEG>(cam, op, px, py, inside, o, d, Y, valid);
+
+  const int lane = threadIdx.x & 31;
+  WarpRays &rays = reinterpret_cast<WarpRays *>(s_kb + 6 * K * nt)[threadIdx.x >> 5];
+  warp_rays1(op, px, py, o, d, valid, lane, &rays);
 
   float T = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f;
   int nbuf = 0;
@@ -260,8 +264,12 @@ __global__ void __launch_bounds__(512, 1) k_composite_fwd_kbuffer(const __grid_c
     }
     stage_sh<NC>(sc, s_idx, nb, s_sh);
     __syncthreads();
-    if (done) continue;
-    for (int b = 0; b < nb && !done; ++b) {
+    for (int c0 = 0; c0 < nb; c0 += 32) {
+    if (__all_sync(kFull, done)) break;
+    unsigned m = near_mask<RS>(s_geo, c0, nb, rays, lane);
+    while (m && !done) {
+      const int b = c0 + __ffs(m) - 1;
+      m &= m - 1;
       float3 og, dg;
       float dd, a;
       if (!eval_response<RS, false>(s_geo[b], px, py, o, d, og, dg, dd, a, op)) continue;
@@ -287,6 +295,7 @@ __global__ void __launch_bounds__(512, 1) k_composite_fwd_kbuffer(const __grid_c
         kb_tau[bi * nt] = tau; kb_a[bi * nt] = al;
         kb_r[bi * nt] = r0; kb_g[bi * nt] = r1; kb_b[bi * nt] = r2; kb_p[bi * nt] = pos;
       }
+    }
     }
   }
   // end of the list: the remaining hits in ascending (tau_max, arrival)
@@ -399,7 +408,7 @@ void fwd_launch(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, con
                 const uint32_t *ranges, unsigned long long *stats, const TileSched &ts, cudaStream_t s) {
   if (op.kbuffer > 0) {
     const int threads = op.tile_w * op.tile_h;
-    const size_t smem = sizeof(float) * 6 * (size_t)op.kbuffer * threads;
+    const size_t smem = sizeof(float) * 6 * (size_t)op.kbuffer * threads + sizeof(WarpRays) * (threads / 32);
     cudaFuncSetAttribute(k_composite_fwd_kbuffer<DEG, RS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaFuncSetAttribute(k_composite_fwd_kbuffer<DEG, RS>, cudaFuncAttributePreferredSharedMemoryCarveout,
                          cudaSharedmemCarveoutMaxShared);
@@ -422,26 +431,30 @@ void fwd_launch(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, con
 
 }  // namespace
 
-// Predicts each tile's walk, orders the tiles longest first, then composites them in that order.
+// Predicts each tile's walk and orders the tiles longest first (into sched, carve_tile_sched).
+ut_status launch_walk_order(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, const uint32_t *vals,
+                            const uint32_t *ranges, void *sched, cudaStream_t s) {
+  const TileSched ts = carve_tile_sched(sched, bd.total_tiles);
+  if (cudaMemsetAsync(ts.hist, 0, sizeof(uint32_t) * (2 * kOrderBuckets + 1), s) != cudaSuccess) return UT_ERR_CUDA;
+  k_fwd_predict<<<(bd.total_tiles + 7) / 8, 256, 0, s>>>(bd, op, reinterpret_cast<const short4 *>(rect), vals,
+                                                         reinterpret_cast<const uint2 *>(ranges), ts);
+  const int ob = (bd.total_tiles + kOrderBuckets - 1) / kOrderBuckets, sms = device_sm_count();
+  k_tile_order<<<ob < sms ? ob : sms, kOrderBuckets, 0, s>>>(bd.total_tiles, ts);
+  count_launches(2);
+  return UT_OK;
+}
+
+// Composites the tiles, longest predicted walk first.
 ut_status launch_composite_fwd(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, const uint32_t *vals,
                                const uint32_t *ranges, unsigned long long *stats, void *sched, cudaStream_t s) {
   if (op.kbuffer > 0 && stats) return UT_ERR_UNSUPPORTED;
   if (bd.total_tiles == 0) return UT_OK;
-  TileSched ts = carve_tile_sched(sched, bd.total_tiles);
   // when every block is resident at once (4 a SM at least, 1 for the k-buffer) the order does not
   // matter: the prediction's launches would only delay the frame
-  const int sms = device_sm_count();
   const long long blocks = (long long)bd.total_tiles * (op.kbuffer > 0 ? 1 : tile_blocks(op));
-  if (blocks <= (op.kbuffer > 0 ? 1 : 4) * sms) {
-    ts.order = nullptr;
-  } else {
-    if (cudaMemsetAsync(ts.hist, 0, sizeof(uint32_t) * (2 * kOrderBuckets + 1), s) != cudaSuccess) return UT_ERR_CUDA;
-    k_fwd_predict<<<(bd.total_tiles + 7) / 8, 256, 0, s>>>(bd, op, reinterpret_cast<const short4 *>(rect), vals,
-                                                           reinterpret_cast<const uint2 *>(ranges), ts);
-    const int ob = (bd.total_tiles + kOrderBuckets - 1) / kOrderBuckets;
-    k_tile_order<<<ob < sms ? ob : sms, kOrderBuckets, 0, s>>>(bd.total_tiles, ts);
-    count_launches(2);
-  }
+  TileSched ts = carve_tile_sched(sched, bd.total_tiles);
+  if (blocks <= (op.kbuffer > 0 ? 1 : 4) * device_sm_count()) ts.order = nullptr;
+  else if (ut_status st = launch_walk_order(bd, op, rect, vals, ranges, sched, s); st != UT_OK) return st;
   const bool rs = any_rs(bd);
 #define UT3D_FWD(D)                                                     \
   (rs ? fwd_launch<D, true>(bd, op, rect, vals, ranges, stats, ts, s) \

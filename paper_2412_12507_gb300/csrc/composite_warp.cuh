@@ -229,8 +229,9 @@ __device__ __forceinline__ float3 pick(const f3x2 &v, int h) {
 }
 
 // The WarpRays of the warp's live pixels (every lane calls it; lane 0 writes *out and the caller
-// synchronises the warp).  square: the warp's pixels are an 8 x 8 square (tile_is_8x8).
-__device__ __forceinline__ void warp_rays(const uint32_t (&pk)[2], const f3x2 &o, const f3x2 &d, bool square, int lane,
+// synchronises the warp).  rows: the warp's pixels are an 8 x rows block (8: two pixels a lane,
+// tile_is_8x8; 4: pixel 0 of each lane, tile_pixel's blocks), or 0 for any other layout.
+__device__ __forceinline__ void warp_rays(const uint32_t (&pk)[2], const f3x2 &o, const f3x2 &d, int rows, int lane,
                                           WarpRays *out) {
   WarpRays w;
   const bool l0 = pk[0] != kDead, l1 = pk[1] != kDead;
@@ -241,12 +242,12 @@ __device__ __forceinline__ void warp_rays(const uint32_t (&pk)[2], const f3x2 &o
   w.y0 = __reduce_min_sync(kFull, min(l0 ? b0 : big, l1 ? b1 : big));
   w.y1 = __reduce_max_sync(kFull, max(l0 ? b0 : -1, l1 ? b1 : -1));
   const unsigned v0 = __ballot_sync(kFull, l0), v1 = __ballot_sync(kFull, l1);
-  const bool plane = square && (v0 & v1) == kFull;
+  const bool plane = v0 == kFull && (rows == 4 || (rows == 8 && v1 == kFull));
   const int ref = v0 ? __ffs(v0) - 1 : (v1 ? __ffs(v1) - 1 : 0);
   w.oc = shfl3(pick(o, v0 ? 0 : 1), ref);
-  if (plane) {  // the plane through the square's corner rays
-    const float3 a = shfl3(pick(d, 0), 0), b = shfl3(pick(d, 0), 7), c = shfl3(pick(d, 1), 24),
-                 e = shfl3(pick(d, 1), 31);
+  if (plane) {  // the plane through the block's corner rays
+    const float3 a = shfl3(pick(d, 0), 0), b = shfl3(pick(d, 0), 7), c = shfl3(pick(d, rows == 8), 24),
+                 e = shfl3(pick(d, rows == 8), 31);
     w.dc = make_float3(0.25f * (a.x + b.x + c.x + e.x), 0.25f * (a.y + b.y + c.y + e.y),
                        0.25f * (a.z + b.z + c.z + e.z));
     w.e1 = make_float3(0.25f * (b.x + e.x - a.x - c.x), 0.25f * (b.y + e.y - a.y - c.y),
@@ -258,11 +259,11 @@ __device__ __forceinline__ void warp_rays(const uint32_t (&pk)[2], const f3x2 &o
     w.e1 = w.e2 = make_float3(0.f, 0.f, 0.f);
   }
   float r = 0.f, ro = 0.f, dn = 0.f, on = 0.f;
-  const float s = ((float)(lane & 7) - 3.5f) * (1.f / 3.5f);
+  const float s = ((float)(lane & 7) - 3.5f) * (1.f / 3.5f), hr = 0.5f * (float)(rows - 1);
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     if (!(h ? l1 : l0)) continue;
-    const float t = ((float)((lane >> 3) + 4 * h) - 3.5f) * (1.f / 3.5f);
+    const float t = plane ? ((float)((lane >> 3) + 4 * h) - hr) / hr : 0.f;
     const float3 dh = pick(d, h), oh = pick(o, h);
     const float3 dd = make_float3(dh.x - fmaf(s, w.e1.x, fmaf(t, w.e2.x, w.dc.x)),
                                   dh.y - fmaf(s, w.e1.y, fmaf(t, w.e2.y, w.dc.y)),
@@ -322,6 +323,30 @@ __device__ __forceinline__ bool block_misses(const float4 (&g)[4], const WarpRay
   float slack = on * nm * w.r + 2e-6f * md * (on + nm * (RS ? w.on + w.ro : 0.f));
   if (RS) slack = fmaf(nm * w.ro, md, slack);
   return cc > 1e-30f && lhs > sqrtf(cc) * (slack + sqrtf(g[3].y) * dmax * 1.0001f);
+}
+
+// The entries of [c0, c0 + 32) of a batch of nb records staged by a block that can reach this warp's
+// pixels, as a mask (every lane calls it).
+template <bool RS>
+__device__ __forceinline__ unsigned near_mask(const float4 (*geo)[4], int c0, int nb, const WarpRays &w, int lane) {
+  bool near_ = false;
+  if (c0 + lane < nb) {
+    float4 g[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) g[q] = geo[c0 + lane][q];
+    const int r0 = __float_as_int(g[3].z), r1 = __float_as_int(g[3].w);
+    near_ = rect_near(w, make_short4((short)(r0 & 0xffff), (short)(r0 >> 16), (short)(r1 & 0xffff), (short)(r1 >> 16))) &&
+            !block_misses<RS>(g, w);
+  }
+  return __ballot_sync(kFull, near_);
+}
+
+// The warp's WarpRays when every lane holds one pixel of a tile (tile_pixel).
+__device__ __forceinline__ void warp_rays1(const DevOpts &op, int px, int py, float3 o, float3 d, bool live, int lane,
+                                           WarpRays *out) {
+  const uint32_t pk[2] = {live ? (uint32_t)px | ((uint32_t)py << 16) : kDead, kDead};
+  const f3x2 o2 = {bc(o.x), bc(o.y), bc(o.z)}, d2 = {bc(d.x), bc(d.y), bc(d.z)};
+  warp_rays(pk, o2, d2, op.tile_w % 8 == 0 && op.tile_h % 4 == 0 ? 4 : 0, lane, out);
 }
 
 // ---------------------------------------------------------------- list entries and SH staging

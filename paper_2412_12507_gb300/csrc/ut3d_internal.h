@@ -68,12 +68,16 @@ ut_status launch_composite_fwd(const BatchDesc &bd, const DevOpts &op, const int
 
 // Backward of the batch into the scenes' gradient outputs (accumulators cleared here).
 size_t backward_workspace_bytes(int n, bool kbuffer);  // accumulators, and the k-buffer record table
+// Orders the tiles by the forward's predicted walk, longest first, into sched.
+ut_status launch_walk_order(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, const uint32_t *vals,
+                            const uint32_t *ranges, void *sched, cudaStream_t stream);
+
 // Scratch of a tile schedule (forward or backward) for `tiles` tiles.
 size_t tile_sched_bytes(int tiles);
 ut_status launch_composite_bwd(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, const uint32_t *vals,
                                const uint32_t *ranges, void *sched, cudaStream_t stream);
 // The backward of the per-ray k-buffer compositing (accumulators cleared by the caller).
 ut_status launch_composite_bwd_kbuffer(const BatchDesc &bd, const DevOpts &op, const int16_t *rect,
-                                       const uint32_t *vals, const uint32_t *ranges, cudaStream_t stream);
+                                       const uint32_t *vals, const uint32_t *ranges, void *sched, cudaStream_t stream);
 
 }  // namespace ut3d
