@@ -483,6 +483,148 @@ __global__ void k_gather_widths(int n, const uint32_t *__restrict__ order, const
   }
 }
 
+// The depth stage of a short list (n <= kSmallSort) in one launch of one block: the work of
+// k_depth_init, the four radix passes, k_gather_widths and the scan of the widths.  A short list
+// leaves most of the chip idle either way, and what those twelve launches cost is their launches
+// and the latency of each (about 2.5 us apiece, 30 us of a 230 us frame of 1000 particles).  The
+// keys stay in shared memory; each pass ranks them like k_radix_downsweep (warp-contiguous
+// segments, same-digit lanes by ballots), and a pass whose digit is the same for every key is
+// skipped.  It also clears the tile ranges, which the row stage fills, when they are few.
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallWarps = kSmallThreads / 32;
+constexpr int kSmallIPT = 8;
+constexpr int kSmallSort = kSmallThreads * kSmallIPT;
+constexpr int kSmallTiles = 16384;
+inline size_t small_sort_smem() { return sizeof(uint32_t) * (2 * (size_t)kSmallSort + 256 * (size_t)kSmallWarps); }
+
+__global__ void __launch_bounds__(kSmallThreads, 1)
+    k_depth_small(int n, const float *__restrict__ depth, const uint32_t *__restrict__ ntiles,
+                  const short4 *__restrict__ rect, int tile_w, uint32_t *__restrict__ order, uint32_t *__restrict__ widths,
+                  uint32_t *__restrict__ offs, u64 *__restrict__ total, uint2 *__restrict__ ranges, int tiles) {
+  extern __shared__ uint32_t s_small[];
+  uint32_t *s_k = s_small, *s_v = s_k + kSmallSort, *s_hist = s_v + kSmallSort;  // [kSmallWarps][256]
+  __shared__ u64 s_warp[kSmallWarps];
+  __shared__ uint32_t s_start[256];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int ipt = (n + kSmallThreads - 1) / kSmallThreads;  // keys a thread
+  const uint32_t lt = (1u << lane) - 1u;
+  for (int i = t; i < tiles; i += kSmallThreads) ranges[i] = make_uint2(0u, 0u);
+
+  // exclusive block scan of one value a thread (and the total)
+  auto scan = [&](u64 x, u64 &tot) -> u64 {
+    const u64 inc = warp_incl_scan_u64(x, lane);
+    __syncthreads();
+    if (lane == 31) s_warp[warp] = inc;
+    __syncthreads();
+    const u64 w = s_warp[lane], wi = warp_incl_scan_u64(w, lane);
+    tot = __shfl_sync(0xffffffffu, wi, 31);
+    return __shfl_sync(0xffffffffu, wi - w, warp) + inc - x;
+  };
+
+  uint32_t k[kSmallIPT], v[kSmallIPT];
+  u64 ksum = 0;
+  uint32_t diff = 0, first = 0;
+#pragma unroll
+  for (int i = 0; i < kSmallIPT; ++i) {
+    const int p = (warp * ipt + i) * 32 + lane;
+    k[i] = 0xffffffffu;
+    v[i] = (uint32_t)p;
+    if (i < ipt && p < n) {
+      const uint32_t nt = ntiles[p];
+      if (nt) k[i] = __float_as_uint(depth[p]);
+      ksum += nt;
+    }
+    if (i == 0) first = k[0];
+    if (i < ipt) diff |= k[i] ^ first;
+  }
+  // bits in which any two keys of the block differ (padding keys past n count like culled ones)
+  if (t == 0) s_start[0] = first;
+  __syncthreads();
+  diff |= first ^ s_start[0];
+  u64 K;
+  scan(ksum, K);
+  if (t == 0) total[1] = K;
+  if (t == 0) s_hist[0] = 0;
+  __syncthreads();
+  diff = __reduce_or_sync(0xffffffffu, diff);
+  if (lane == 0) atomicOr(&s_hist[0], diff);
+  __syncthreads();
+  diff = s_hist[0];
+  for (int shift = 0; shift < 32; shift += 8) {
+    if (((diff >> shift) & 255u) == 0) continue;  // block-uniform
+    __syncthreads();
+    uint32_t *wh = s_hist + 256 * warp;
+    for (int d = lane; d < 256; d += 32) wh[d] = 0;
+    __syncwarp();
+    uint32_t rank[kSmallIPT];
+#pragma unroll
+    for (int i = 0; i < kSmallIPT; ++i) {
+      if (i >= ipt) break;
+      const uint32_t d = (k[i] >> shift) & 255u, peers = digit_peers(d);
+      const int leader = __ffs(peers) - 1;
+      uint32_t before = 0;
+      if (lane == leader) before = atomicAdd(&wh[d], (uint32_t)__popc(peers));
+      rank[i] = __shfl_sync(0xffffffffu, before, leader) + (uint32_t)__popc(peers & lt);
+    }
+    __syncthreads();
+    uint32_t sum = 0;
+    if (t < 256) {
+      for (int w = 0; w < kSmallWarps; ++w) {
+        const uint32_t c = s_hist[256 * w + t];
+        s_hist[256 * w + t] = sum;
+        sum += c;
+      }
+    }
+    u64 tot;
+    const u64 ex = scan(sum, tot);
+    if (t < 256) s_start[t] = (uint32_t)ex;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kSmallIPT; ++i) {
+      if (i >= ipt) break;
+      const uint32_t d = (k[i] >> shift) & 255u, pos = s_start[d] + wh[d] + rank[i];
+      s_k[pos] = k[i];
+      s_v[pos] = v[i];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kSmallIPT; ++i) {
+      if (i >= ipt) break;
+      const int p = (warp * ipt + i) * 32 + lane;
+      k[i] = s_k[p];
+      v[i] = s_v[p];
+    }
+  }
+  // tile columns of each particle in depth order, and their exclusive scan (the n particles come
+  // before the padding: a stable order, and no key exceeds the padding's)
+  uint32_t carry = 0;
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < kSmallIPT; ++i) {
+    if (i >= ipt) break;
+    const int p = (warp * ipt + i) * 32 + lane;
+    uint32_t w = 0;
+    if (p < n) {
+      order[p] = v[i];
+      if (ntiles[v[i]]) {
+        const short4 r = rect[v[i]];
+        w = (uint32_t)(r.z / tile_w - r.x / tile_w + 1);
+      }
+      widths[p] = w;
+    }
+    s_k[p] = w;
+  }
+  __syncthreads();
+  for (int base = 0; base < ipt * kSmallThreads; base += kSmallThreads) {
+    u64 tot;
+    const uint32_t w = s_k[base + t];
+    const u64 ex = scan(w, tot);
+    if (base + t < n) offs[base + t] = carry + (uint32_t)ex;
+    carry += (uint32_t)tot;
+  }
+  if (t == 0) total[0] = carry;
+}
+
 __global__ void k_write_kout(const u64 *__restrict__ total, int64_t *__restrict__ k_out) { *k_out = (int64_t)*total; }
 
 // Lane owning output position p among the warp's 32 consecutive runs (run l starts at
@@ -1227,15 +1369,30 @@ ut_status launch_bin(const BatchDesc &bd, const float *depth, const int16_t *rec
     ~GuardCheck() { k_check_guards<<<1, 256, 0, s>>>(static_cast<const unsigned char *>(ws), b.guards); }
   } guard_check{b, ws, s};
 #endif
-  if (cudaMemsetAsync(ranges, 0, sizeof(uint32_t) * 2 * (size_t)tiles, s) != cudaSuccess) return UT_ERR_CUDA;
-  if (cudaMemsetAsync(b.total, 0, 2 * sizeof(u64), s) != cudaSuccess) return UT_ERR_CUDA;
+  // a short single-view list: one launch for the depth stage (batches keep one launch sequence)
+  const bool small = short_sort && n > 0 && n <= kSmallSort;
+  const bool clear = !small || tiles > kSmallTiles;
+  if (clear && cudaMemsetAsync(ranges, 0, sizeof(uint32_t) * 2 * (size_t)tiles, s) != cudaSuccess) return UT_ERR_CUDA;
+  if (!small && cudaMemsetAsync(b.total, 0, 2 * sizeof(u64), s) != cudaSuccess) return UT_ERR_CUDA;
   if (n > 0) {
     const int g = grid_for(n, kThreads);
     const Count cn{nullptr, 0, (uint32_t)n};
-    // depth keys, and K = sum of ntiles (reported even when it exceeds the capacity)
-    k_depth_init<<<g, kThreads, 0, s>>>(n, depth, ntiles, b.dk[0], b.dv[0], b.total + 1);
-    count_launches(1);
-    const int r = radix_sort(b.dk, b.dv, cn, (u64)n, 0, 32, b.spine, b.chunk, s, short_sort);
+    int r = 0;  // the buffer of b.dv that holds the depth order
+    if (small) {
+      const size_t smem = small_sort_smem();
+      if (cudaFuncSetAttribute(k_depth_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return UT_ERR_CUDA;
+      k_depth_small<<<1, kSmallThreads, smem, s>>>(n, depth, ntiles, r4, op.tile_w, b.dv[0], b.cnt, b.offs, b.total,
+                                                   reinterpret_cast<uint2 *>(ranges), clear ? 0 : tiles);
+      count_launches(1);
+    } else {
+      // depth keys, and K = sum of ntiles (reported even when it exceeds the capacity)
+      k_depth_init<<<g, kThreads, 0, s>>>(n, depth, ntiles, b.dk[0], b.dv[0], b.total + 1);
+      r = radix_sort(b.dk, b.dv, cn, (u64)n, 0, 32, b.spine, b.chunk, s, short_sort);
+      k_gather_widths<<<g, kThreads, 0, s>>>(n, b.dv[r], ntiles, r4, op.tile_w, b.cnt);
+      count_launches(2);
+      scan(b.cnt, b.offs, cn, (u64)n, b.chunk, b.total, s);
+    }
     // buffer plan: column keys ping-pong in x[0] / x[1]; values (column, then row) over x[2]
     // and the caller's vals, arranged so that the row stage lands in vals: the row scatter
     // reads the column values from x[2]; the row radix passes end in vals
@@ -1248,9 +1405,6 @@ ut_status launch_bin(const BatchDesc &bd, const float *depth, const int16_t *rec
     cv[0] = (cp & 1) ? (scatter ? r1 : r0) : (scatter ? r0 : r1);  // column values end in x[2] / r1
     cv[1] = cv[0] == r0 ? r1 : r0;
     // 2. column entries in depth order, sorted by global tile column
-    k_gather_widths<<<g, kThreads, 0, s>>>(n, b.dv[r], ntiles, r4, op.tile_w, b.cnt);
-    count_launches(1);
-    scan(b.cnt, b.offs, cn, (u64)n, b.chunk, b.total, s);
     const Count cc{b.total, (u64)cap, 0, b.total + 1};  // nothing is written unless K fits
     const int eg = (int)std::min<u64>((u64)(n + kThreads - 1) / kThreads, (u64)device_sm_count() * 16);
     if (scatter)
