@@ -269,11 +269,15 @@ __device__ __forceinline__ uint32_t digit_peers(uint32_t d) {
   return peers;
 }
 
-// Per radix tile, the count of each digit (digit-major layout counts[d * nb + b]).  Keys are
-// read as uint4 (the next tile's while the current one is counted into the warps' shared
-// histograms and totalled).
+// Per radix tile, the count of each digit: digit-major (counts[d * nb + b]) for the scanned spine, or,
+// with group (the short sort), tile-major (counts[b * 256 + d]) with the totals of each kGroup
+// consecutive tiles added to group[(b / kGroup) * 256 + d].  Keys are read as uint4 (the next
+// tile's while the current one is counted into the warps' shared histograms and totalled).
+constexpr uint32_t kGroup = 16;
+
 __global__ void __launch_bounds__(kThreads) k_radix_upsweep(const uint32_t *__restrict__ keys, Count cnt, int shift,
-                                                            uint32_t mask, uint32_t *__restrict__ counts) {
+                                                            uint32_t mask, uint32_t *__restrict__ counts,
+                                                            uint32_t *__restrict__ group) {
   __shared__ uint32_t s_wh[kWarps][256];
   const uint32_t n = cnt.get();
   const uint32_t nb = (n + kRTile - 1) / kRTile;
@@ -319,7 +323,12 @@ __global__ void __launch_bounds__(kThreads) k_radix_upsweep(const uint32_t *__re
       uint32_t s = 0;
 #pragma unroll
       for (int w = 0; w < kWarps; ++w) s += s_wh[w][threadIdx.x];
-      counts[(size_t)threadIdx.x * nb + b] = s;
+      if (group) {
+        counts[(size_t)b * 256 + threadIdx.x] = s;
+        if (s) atomicAdd(&group[(b / kGroup) * 256 + threadIdx.x], s);
+      } else {
+        counts[(size_t)threadIdx.x * nb + b] = s;
+      }
     }
     __syncthreads();
   }
@@ -346,17 +355,22 @@ __device__ __forceinline__ void load_radix_tile(const uint32_t *__restrict__ key
 // broadcast), digit starts from the per-warp counts and a block scan, a scatter into shared
 // memory in digit order, and a write-out grouped by digit (coalesced runs).  The next tile's
 // keys, values and global digit offsets are loaded while the current tile is written out.
-// SELF (lists of at most kSelfRadixTiles tiles): `offsets` holds the upsweep's raw digit-major
-// counts and every block derives its own offsets from them (the digit totals' exclusive scan
-// plus the counts of its digit in the tiles before it), which saves the two scan launches.
-constexpr uint32_t kSelfRadixTiles = 128;
+// SELF (lists of at most kSelfRadixTiles tiles): `offsets` holds the upsweep's raw tile-major
+// counts and every block derives its own offsets from them and the group totals (the digit
+// totals' exclusive scan, plus its digit's totals in the groups before its tile's and counts in
+// the group's tiles before it: at most nb / 16 + 15 coalesced loads a thread), which saves the two
+// scan launches (bin_and_sort of 300k particles at 1920x1080: 182 us with four launches a pass,
+// 153 with two).  1024 tiles (2M keys): 79 loads of a kilobyte row for a tile of 16 KB; beyond, they
+// would outgrow the two scans, which cost about 8 us.
+constexpr uint32_t kSelfRadixTiles = 1024;
 
 template <bool SELF>
 __global__ void __launch_bounds__(kThreads) k_radix_downsweep(const uint32_t *__restrict__ keys_in,
                                                               const uint32_t *__restrict__ vals_in,
                                                               uint32_t *__restrict__ keys_out,
                                                               uint32_t *__restrict__ vals_out, Count cnt, int shift,
-                                                              uint32_t mask, const uint32_t *__restrict__ offsets) {
+                                                              uint32_t mask, const uint32_t *__restrict__ offsets,
+                                                              const uint32_t *__restrict__ group) {
   __shared__ uint32_t s_k[kRTile];
   __shared__ uint32_t s_v[kRTile];
   __shared__ uint32_t s_whist[kWarps][256];
@@ -373,8 +387,11 @@ __global__ void __launch_bounds__(kThreads) k_radix_downsweep(const uint32_t *__
   __shared__ uint32_t s_dbase[SELF ? 256 : 1];
   if (SELF) {  // exclusive scan of the digit totals
     uint32_t t = 0;
-    if (threadIdx.x < nd)
-      for (uint32_t bb = 0; bb < nb; ++bb) t += offsets[(size_t)threadIdx.x * nb + bb];
+    const uint32_t ng = (nb + kGroup - 1) / kGroup;
+    if (threadIdx.x < nd) {
+#pragma unroll 8
+      for (uint32_t g = 0; g < ng; ++g) t += group[g * 256 + threadIdx.x];
+    }
     u64 ex;
     block_excl_scan_u64(t, s_warp, ex);
     if (threadIdx.x < nd) s_dbase[threadIdx.x] = (uint32_t)ex;
@@ -385,7 +402,11 @@ __global__ void __launch_bounds__(kThreads) k_radix_downsweep(const uint32_t *__
     if (threadIdx.x >= nd) return 0u;
     if (!SELF) return offsets[(size_t)threadIdx.x * nb + bb];
     uint32_t o = s_dbase[SELF ? threadIdx.x : 0];
-    for (uint32_t b2 = 0; b2 < bb; ++b2) o += offsets[(size_t)threadIdx.x * nb + b2];
+    const uint32_t g1 = bb / kGroup;
+#pragma unroll 8
+    for (uint32_t g = 0; g < g1; ++g) o += group[g * 256 + threadIdx.x];
+#pragma unroll 4
+    for (uint32_t b2 = g1 * kGroup; b2 < bb; ++b2) o += offsets[(size_t)b2 * 256 + threadIdx.x];
     return o;
   };
   uint32_t k[kRIPT], v[kRIPT];
@@ -451,13 +472,15 @@ __global__ void __launch_bounds__(kThreads) k_radix_downsweep(const uint32_t *__
 // ---------------------------------------------------------------- binning kernels
 
 // Depth keys (culled particles last) and the particle indices, and K = sum of ntiles added to
-// *ksum (zeroed beforehand) with one atomic per block.
+// *ksum (zeroed beforehand) with one atomic per block; clears the short passes' group totals.
 __global__ void __launch_bounds__(kThreads) k_depth_init(int n, const float *__restrict__ depth,
                                                          const uint32_t *__restrict__ ntiles,
                                                          uint32_t *__restrict__ dk, uint32_t *__restrict__ dv,
-                                                         u64 *__restrict__ ksum) {
+                                                         u64 *__restrict__ ksum, uint32_t *__restrict__ group,
+                                                         int words) {
   __shared__ u64 s_warp[kWarps + 1];
   u64 k = 0;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < words; i += gridDim.x * blockDim.x) group[i] = 0u;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const uint32_t t = ntiles[i];
     dk[i] = t > 0 ? __float_as_uint(depth[i]) : 0xffffffffu;
@@ -500,7 +523,8 @@ inline size_t small_sort_smem() { return sizeof(uint32_t) * (2 * (size_t)kSmallS
 __global__ void __launch_bounds__(kSmallThreads, 1)
     k_depth_small(int n, const float *__restrict__ depth, const uint32_t *__restrict__ ntiles,
                   const short4 *__restrict__ rect, int tile_w, uint32_t *__restrict__ order, uint32_t *__restrict__ widths,
-                  uint32_t *__restrict__ offs, u64 *__restrict__ total, uint2 *__restrict__ ranges, int tiles) {
+                  uint32_t *__restrict__ offs, u64 *__restrict__ total, uint2 *__restrict__ ranges, int tiles,
+                  uint32_t *__restrict__ group, int words) {
   extern __shared__ uint32_t s_small[];
   uint32_t *s_k = s_small, *s_v = s_k + kSmallSort, *s_hist = s_v + kSmallSort;  // [kSmallWarps][256]
   __shared__ u64 s_warp[kSmallWarps];
@@ -509,6 +533,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
   const int ipt = (n + kSmallThreads - 1) / kSmallThreads;  // keys a thread
   const uint32_t lt = (1u << lane) - 1u;
   for (int i = t; i < tiles; i += kSmallThreads) ranges[i] = make_uint2(0u, 0u);
+  for (int i = t; i < words; i += kSmallThreads) group[i] = 0u;
 
   // exclusive block scan of one value a thread (and the total)
   auto scan = [&](u64 x, u64 &tot) -> u64 {
@@ -870,9 +895,9 @@ __global__ void k_col_bounds(const uint32_t *__restrict__ ckeys, Count cc, uint3
 // The chunk plan from the column bounds (one block of 1024 threads).  With dspine, the column
 // order came from one radix pass over all column bits, and the bounds are read off its scanned
 // digit-major counts instead (column c starts at dspine[c * tiles], tiles = radix tiles of the
-// M column entries) and written to colb here; with raw, dspine holds the pass's unscanned
-// counts (the short pass derived its offsets itself) and the bounds come from the exclusive
-// scan of the per-column totals.
+// M column entries) and written to colb here; with raw, dspine holds the short pass's group totals
+// (it derived its offsets itself) and the bounds come from the exclusive scan of the per-column
+// totals.
 __global__ void __launch_bounds__(1024) k_chunk_plan(const __grid_constant__ BatchDesc bd, uint32_t *__restrict__ colb,
                                                      ChunkPlan pl, const uint32_t *__restrict__ dspine, int ndigits,
                                                      Count mcnt, int raw) {
@@ -889,13 +914,13 @@ __global__ void __launch_bounds__(1024) k_chunk_plan(const __grid_constant__ Bat
     }
     __syncthreads();
   } else if (dspine) {
-    const uint32_t M = mcnt.get(), nt = (M + kRTile - 1) / kRTile;
+    const uint32_t M = mcnt.get(), ng = (M + kRTile * kGroup - 1) / (kRTile * kGroup);
     u64 carry = 0;
     for (int c0 = 0; c0 < cols; c0 += 1024) {
       const int c = c0 + t;
       uint32_t tot = 0;
       if (c < cols)
-        for (uint32_t tt = 0; tt < nt; ++tt) tot += dspine[(size_t)c * nt + tt];
+        for (uint32_t g = 0; g < ng; ++g) tot += dspine[g * 256 + c];
       const u64 inc = warp_incl_scan_u64((u64)tot, lane);
       if (lane == 31) s_w[warp] = inc;
       __syncthreads();
@@ -1311,25 +1336,29 @@ void scan(const uint32_t *in, uint32_t *out, L len, u64 max_len, u64 *chunk, u64
 
 // Sorts (keys, vals) in place across the two buffers; returns the buffer index holding the result.
 // Bits [shift0, shift0 + bits) of the keys are sorted.  With self_offsets, lists of at most
-// kSelfRadixTiles radix tiles skip the spine scan (the downsweep derives its offsets; the spine
-// is then left unscanned, so callers that read it afterwards pass false).
+// kSelfRadixTiles radix tiles skip the spine scan (the downsweep derives its offsets from the
+// group totals, cleared beforehand, one array of group_words(max_count) a pass from `group`; the
+// spine is then left unscanned, so callers that read it afterwards pass null).
+inline size_t group_words(u64 count) { return 256 * (size_t)ceil_div(ceil_div(count, kRTile), kGroup); }
+
 int radix_sort(uint32_t *keys[2], uint32_t *vals[2], Count cnt, u64 max_count, int shift0, int bits,
-               uint32_t *spine, u64 *chunk, cudaStream_t s, bool self_offsets = false) {
+               uint32_t *spine, u64 *chunk, cudaStream_t s, uint32_t *group = nullptr) {
   int cur = 0;
   int g = grid_for(max_count, kRTile);
-  const bool self = self_offsets && ceil_div(max_count, kRTile) <= kSelfRadixTiles;
+  const bool self = group && ceil_div(max_count, kRTile) <= kSelfRadixTiles;
   for (int shift = shift0; shift < shift0 + bits; shift += kRadixBits) {
     int db = shift0 + bits - shift < kRadixBits ? shift0 + bits - shift : kRadixBits;
     uint32_t mask = (1u << db) - 1u;
-    k_radix_upsweep<<<g, kThreads, 0, s>>>(keys[cur], cnt, shift, mask, spine);
+    k_radix_upsweep<<<g, kThreads, 0, s>>>(keys[cur], cnt, shift, mask, spine, self ? group : nullptr);
     if (self) {
       k_radix_downsweep<true><<<g, kThreads, 0, s>>>(keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], cnt, shift,
-                                                    mask, spine);
+                                                    mask, spine, group);
+      group += group_words(max_count);
     } else {
       SpineLen sl{cnt, (int)mask + 1};
       scan(spine, spine, sl, (u64)(mask + 1) * ceil_div(max_count, kRTile), chunk, nullptr, s);
       k_radix_downsweep<false><<<g, kThreads, 0, s>>>(keys[cur], vals[cur], keys[cur ^ 1], vals[cur ^ 1], cnt,
-                                                     shift, mask, spine);
+                                                     shift, mask, spine, nullptr);
     }
     count_launches(2);
     cur ^= 1;
@@ -1371,6 +1400,20 @@ ut_status launch_bin(const BatchDesc &bd, const float *depth, const int16_t *rec
 #endif
   // a short single-view list: one launch for the depth stage (batches keep one launch sequence)
   const bool small = short_sort && n > 0 && n <= kSmallSort;
+  // Short passes of the single-view call (radix_sort): their group totals live in the row stage's
+  // spine, which nothing else uses until the column order is done, and are cleared by the depth
+  // stage's first kernel.  Column pass: the buffer plan below.
+  const bool scatter = max_rows <= kScatterMaxRows && bd.total_cols <= kScatterMaxCols;
+  const int cbits = bits_for(bd.total_cols), rbits = bits_for(bd.total_rows);
+  const int cp = (cbits + kRadixBits - 1) / kRadixBits, rp = (rbits + kRadixBits - 1) / kRadixBits;
+  const size_t room = plan_spine_words(max_rows, tiles, bd.total_cols);
+  const bool depth_short = short_sort && !small && 4 * group_words((u64)n) <= room &&
+                           ceil_div((u64)n, kRTile) <= kSelfRadixTiles;
+  const size_t gdepth = depth_short ? 4 * group_words((u64)n) : 0;
+  const bool col_short = short_sort && scatter && cp == 1 && ceil_div((u64)cap, kRTile) <= kSelfRadixTiles &&
+                         gdepth + group_words((u64)cap) <= room;
+  uint32_t *const group = b.tspine;
+  const size_t gtotal = gdepth + (col_short ? group_words((u64)cap) : 0);
   const bool clear = !small || tiles > kSmallTiles;
   if (clear && cudaMemsetAsync(ranges, 0, sizeof(uint32_t) * 2 * (size_t)tiles, s) != cudaSuccess) return UT_ERR_CUDA;
   if (!small && cudaMemsetAsync(b.total, 0, 2 * sizeof(u64), s) != cudaSuccess) return UT_ERR_CUDA;
@@ -1383,12 +1426,12 @@ ut_status launch_bin(const BatchDesc &bd, const float *depth, const int16_t *rec
       if (cudaFuncSetAttribute(k_depth_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return UT_ERR_CUDA;
       k_depth_small<<<1, kSmallThreads, smem, s>>>(n, depth, ntiles, r4, op.tile_w, b.dv[0], b.cnt, b.offs, b.total,
-                                                   reinterpret_cast<uint2 *>(ranges), clear ? 0 : tiles);
+                                                   reinterpret_cast<uint2 *>(ranges), clear ? 0 : tiles, group, (int)gtotal);
       count_launches(1);
     } else {
       // depth keys, and K = sum of ntiles (reported even when it exceeds the capacity)
-      k_depth_init<<<g, kThreads, 0, s>>>(n, depth, ntiles, b.dk[0], b.dv[0], b.total + 1);
-      r = radix_sort(b.dk, b.dv, cn, (u64)n, 0, 32, b.spine, b.chunk, s, short_sort);
+      k_depth_init<<<g, kThreads, 0, s>>>(n, depth, ntiles, b.dk[0], b.dv[0], b.total + 1, group, (int)gtotal);
+      r = radix_sort(b.dk, b.dv, cn, (u64)n, 0, 32, b.spine, b.chunk, s, depth_short ? group : nullptr);
       k_gather_widths<<<g, kThreads, 0, s>>>(n, b.dv[r], ntiles, r4, op.tile_w, b.cnt);
       count_launches(2);
       scan(b.cnt, b.offs, cn, (u64)n, b.chunk, b.total, s);
@@ -1396,9 +1439,6 @@ ut_status launch_bin(const BatchDesc &bd, const float *depth, const int16_t *rec
     // buffer plan: column keys ping-pong in x[0] / x[1]; values (column, then row) over x[2]
     // and the caller's vals, arranged so that the row stage lands in vals: the row scatter
     // reads the column values from x[2]; the row radix passes end in vals
-    const bool scatter = max_rows <= kScatterMaxRows && bd.total_cols <= kScatterMaxCols;
-    const int cbits = bits_for(bd.total_cols), rbits = bits_for(bd.total_rows);
-    const int cp = (cbits + kRadixBits - 1) / kRadixBits, rp = (rbits + kRadixBits - 1) / kRadixBits;
     uint32_t *r0 = (scatter || (rp & 1)) ? b.x[2] : vals;  // row values start here ...
     uint32_t *r1 = r0 == vals ? b.x[2] : vals;               // ... and end in vals
     uint32_t *cv[2], *ck[2] = {b.x[0], b.x[1]};
@@ -1414,16 +1454,16 @@ ut_status launch_bin(const BatchDesc &bd, const float *depth, const int16_t *rec
       k_emit_cols<false><<<eg, kThreads, 0, s>>>(bd, n, b.dv[r], b.offs, b.cnt, r4, cc, op.tile_w, op.tile_h, ck[0],
                                                  cv[0]);
     count_launches(1);
-    // the short pass leaves the spine unscanned: only the single-pass scatter path reads it, raw
-    const bool col_short = short_sort && scatter && cp == 1 && ceil_div((u64)cap, kRTile) <= kSelfRadixTiles;
-    const int rc = radix_sort(ck, cv, cc, (u64)cap, 0, cbits, b.spine, b.chunk, s, col_short);
+    const int rc = radix_sort(ck, cv, cc, (u64)cap, 0, cbits, b.spine, b.chunk, s,
+                              col_short ? group + gdepth : nullptr);
     const Count ck2{b.total + 1, (u64)cap, 0};
     if (scatter) {
       // 3. row entries scattered straight into (tile, depth) order
       const uint32_t *ckc = ck[rc], *cvc = cv[rc];
       const int blocks = (kChunkWarps + bd.total_cols + kWarps - 1) / kWarps;
       if (cp == 1) {  // bounds from the single column pass's digit counts
-        k_chunk_plan<<<1, 1024, 0, s>>>(bd, b.colb, b.plan, b.spine, 1 << cbits, cc, col_short ? 1 : 0);
+        k_chunk_plan<<<1, 1024, 0, s>>>(bd, b.colb, b.plan, col_short ? group + gdepth : b.spine, 1 << cbits, cc,
+                                          col_short ? 1 : 0);
       } else {
         if (cudaMemsetAsync(b.colb, 0, sizeof(uint32_t) * 2 * (size_t)bd.total_cols, s) != cudaSuccess)
           return UT_ERR_CUDA;
