@@ -15,13 +15,20 @@
 // unclamped channels) go to the particle's accumulators.  The lanes of a warp blend in step (one
 // blend event per lane per staged particle, and per step of the final drain), and the events of a
 // step are grouped by particle: neighbouring pixels' buffers evolve alike, so a step's 20 or so
-// events name three or four particles.  A group of four or more lanes sums its contributions with
-// reduce-scatters over the warp and adds each value with one atomic; the lanes of smaller groups
-// add their own, one global atomic per value (a window of
-// per-list-position accumulators in shared memory was measured 5x slower: the lanes of a warp
-// blend the same particle at nearly the same time, and shared-memory atomics on one address
-// serialise, while the L2's reductions absorb them).
+// events name three or four particles.  The groups' SH gradients are contracted on the tensor
+// cores, D[basis][(group, channel)] = sum over the warp's pixels of Y g_c w, two groups at a time:
+// m16n8k16 BF16 with both operands split in three (24 bits, the six leading cross terms, FP32
+// accumulation; errors against the FP64 oracle equal to those of the FP32 shuffles it replaced:
+// SH 1.07e-6 / 1.07e-6, 7.5e-7 / 7.4e-7).  The 13 geometry partials of a group of four or more
+// lanes are summed with a reduce-scatter, those of a smaller one added lane by lane.  Bound by
+// instruction issue and the latency of two blocks an SM; SH by three reduce-scatters a group cost
+// 1750 us where this costs 1207 (100k particles, 1280x720, k = 16).
+// (A window of per-list-position accumulators in shared memory was measured 5x slower: the lanes
+// of a warp blend the same particle at nearly the same time, and shared-memory atomics on one
+// address serialise, while the L2's reductions absorb them.)
 // Selection by tau_max is piecewise constant and carries no gradient.
+#include <cuda_bf16.h>
+
 #include "composite_warp.cuh"
 
 namespace ut3d {
@@ -43,6 +50,27 @@ __device__ __forceinline__ void kb_reduce_scatter16(float (&v)[16], int lane) {
     }
   }
   v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// Two floats as three bf16 pairs (x = hi + mid + lo to 24 bits).
+__device__ __forceinline__ void split3_bf16x2(float x, float y, uint32_t &hi, uint32_t &mid, uint32_t &lo) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+  const float2 hf = __bfloat1622float2(h);
+  const float rx = x - hf.x, ry = y - hf.y;
+  const __nv_bfloat162 m = __floats2bfloat162_rn(rx, ry);
+  const float2 mf = __bfloat1622float2(m);
+  const __nv_bfloat162 l = __floats2bfloat162_rn(rx - mf.x, ry - mf.y);
+  hi = *reinterpret_cast<const uint32_t *>(&h);
+  mid = *reinterpret_cast<const uint32_t *>(&m);
+  lo = *reinterpret_cast<const uint32_t *>(&l);
+}
+
+// D += A B for one m16n8k16 BF16 tile (FP32 accumulate).
+__device__ __forceinline__ void kb_mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
 // The record table of the scene's particles: M (row-major, 9), M mu, mu and sigma, 16 floats.
@@ -72,7 +100,7 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
   __shared__ float4 s_aux[kBatchKB];
   __shared__ __align__(16) float s_sh[kBatchKB * NC];
   __shared__ uint32_t s_idx[kBatchKB];
-  extern __shared__ __align__(16) float s_kb[];  // [6][k][threads]: tau, alpha, r, g, b, list position; [warps] rays
+  extern __shared__ __align__(16) float s_kb[];  // [6][k][threads]: tau, alpha, r, g, b, list position; [warps] rays; [warps][3][32]
 
   const int tile = (int)(ts.order ? ts.order[blockIdx.x] : blockIdx.x);
   const DevView &view = bd.v[view_of_tile(bd, tile)];
@@ -186,17 +214,92 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
   const int lane = threadIdx.x & 31;
   WarpRays &rays = reinterpret_cast<WarpRays *>(s_kb + 6 * K * nt)[threadIdx.x >> 5];
   warp_rays1(op, px, py, o, d, valid, lane, &rays);
+  const int g8 = lane >> 2, t4 = lane & 3;
+  float *s_gc = s_kb + 6 * K * nt + (sizeof(WarpRays) / 4) * (nt / 32) + 96 * (threadIdx.x >> 5);  // [3][32]
+  // A operand of emit's contraction (basis functions x the warp's 32 pixels), fixed for the tile:
+  // fragment r of k-step ks holds basis g8 (+8 for odd r) at pixels 16 ks + 2 t4 + {0, 1} (+8 for r >= 2)
+  uint32_t A[2][3][4];  // [k-step][hi, mid, lo][fragment]
+#pragma unroll
+  for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int p = 16 * ks + 2 * t4 + (r >= 2 ? 8 : 0), kk = g8 + (r & 1 ? 8 : 0);
+      float y0 = 0.f, y1 = 0.f;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        constexpr int n = NSH;
+        const int src = k + (r & 1 ? 8 : 0);
+        if (src >= n) continue;
+        const float u0 = __shfl_sync(kFull, Y[src < n ? src : 0], p), u1 = __shfl_sync(kFull, Y[src < n ? src : 0], p + 1);
+        if (kk == src) {
+          y0 = u0;
+          y1 = u1;
+        }
+      }
+      split3_bf16x2(y0, y1, A[ks][0][r], A[ks][1][r], A[ks][2][r]);
+    }
+
   auto emit = [&]() {
-    const unsigned act = __ballot_sync(0xffffffffu, has_ev);
+    const unsigned act = __ballot_sync(kFull, has_ev);
     if (!act) return;
-    const unsigned grp = __match_any_sync(0xffffffffu, has_ev ? ev_idx : 0xffffffffu);
-    unsigned big = __ballot_sync(0xffffffffu, has_ev && (int)(__ffs(grp) - 1) == lane && __popc(grp) >= 4);
+    const unsigned grp = __match_any_sync(kFull, has_ev ? ev_idx : 0xffffffffu);
+    const bool leader = has_ev && __ffs(grp) - 1 == lane;
+    // SH: D[basis][column] = sum over pixels of Y g_c w, columns (group, channel), two groups at a
+    // time.  A lane's column is g8 (channel g8 mod 3); its pixel pairs are split once a step and
+    // masked by the column's group.
+    __syncwarp();
+#pragma unroll
+    for (int c = 0; c < 3; ++c) s_gc[32 * c + lane] = has_ev ? ev_gc[c] : 0.f;
+    __syncwarp();
+    uint32_t B[4][3];  // pixel pairs 2 t4 + {0, 8, 16, 24}
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float2 w = *reinterpret_cast<const float2 *>(s_gc + 32 * (g8 % 3) + 8 * q + 2 * t4);
+      split3_bf16x2(w.x, w.y, B[q][0], B[q][1], B[q][2]);
+    }
+    unsigned rem = __ballot_sync(kFull, leader);
+    const unsigned big0 = __ballot_sync(kFull, leader && __popc(grp) >= 4);
+    while (rem) {
+      const int la = __ffs(rem) - 1;
+      rem &= rem - 1;
+      const int lb = rem ? __ffs(rem) - 1 : -1;
+      rem &= rem - 1;
+      const unsigned ga = __shfl_sync(kFull, grp, la), gb = lb >= 0 ? __shfl_sync(kFull, grp, lb) : 0u;
+      const uint32_t ia = __shfl_sync(kFull, ev_idx, la), ib = __shfl_sync(kFull, ev_idx, lb >= 0 ? lb : la);
+      const unsigned cm = (g8 < 3 ? ga : (g8 < 6 ? gb : 0u)) >> (2 * t4);
+      float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int ks = 0; ks < 2; ++ks) {
+        uint32_t b[2][3];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const unsigned two = cm >> (16 * ks + 8 * j);
+          const uint32_t msk = (two & 1u ? 0xffffu : 0u) | (two & 2u ? 0xffff0000u : 0u);
+#pragma unroll
+          for (int q = 0; q < 3; ++q) b[j][q] = B[2 * ks + j][q] & msk;
+        }
+        kb_mma(acc, A[ks][0], b[0][2], b[1][2]);  // smallest terms first
+        kb_mma(acc, A[ks][2], b[0][0], b[1][0]);
+        kb_mma(acc, A[ks][1], b[0][1], b[1][1]);
+        kb_mma(acc, A[ks][0], b[0][1], b[1][1]);
+        kb_mma(acc, A[ks][1], b[0][0], b[1][0]);
+        kb_mma(acc, A[ks][0], b[0][0], b[1][0]);
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        const int k = g8 + (r >= 2 ? 8 : 0), col = 2 * t4 + (r & 1);
+        if (k < NSH && col < (lb >= 0 ? 6 : 3) && acc[r] != 0.f)
+          atomicAdd(&sc.d_sh[(size_t)(col < 3 ? ia : ib) * NC + 3 * k + (col < 3 ? col : col - 3)], acc[r]);
+      }
+    }
+    // geometry: groups of four or more lanes by reduce-scatter, smaller ones lane by lane
+    unsigned big = big0;
     const int vi = lane >> 1;
     while (big) {
       const int l = __ffs(big) - 1;
       big &= big - 1;
-      const unsigned gm = __shfl_sync(0xffffffffu, grp, l);
-      const uint32_t p0 = __shfl_sync(0xffffffffu, ev_idx, l);
+      const unsigned gm = __shfl_sync(kFull, grp, l);
+      const uint32_t p0 = __shfl_sync(kFull, ev_idx, l);
       const bool in = (gm >> lane) & 1u;
       float v[16];
 #pragma unroll
@@ -209,24 +312,8 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
       v[13] = v[14] = v[15] = 0.f;
       kb_reduce_scatter16(v, lane);
       if (!(lane & 1) && vi < 13) atomicAdd(&sc.gacc[(size_t)p0 * 16 + vi], v[0]);
-#pragma unroll
-      for (int ch = 0; ch < 3; ++ch) {
-        if (!__any_sync(0xffffffffu, in && ev_gc[ch] != 0.f)) continue;
-        float u[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) u[k] = (in && k < NSH) ? ev_gc[ch] * Y[k < NSH ? k : 0] : 0.f;
-        kb_reduce_scatter16(u, lane);
-        if (!(lane & 1) && vi < NSH && u[0] != 0.f) atomicAdd(&sc.d_sh[(size_t)p0 * NC + 3 * vi + ch], u[0]);
-      }
     }
     if (has_ev && __popc(grp) < 4) {
-      float *dsh = sc.d_sh + (size_t)ev_idx * NC;
-#pragma unroll
-      for (int ch = 0; ch < 3; ++ch) {
-        if (ev_gc[ch] == 0.f) continue;
-#pragma unroll
-        for (int k = 0; k < NSH; ++k) atomicAdd(&dsh[3 * k + ch], ev_gc[ch] * Y[k]);
-      }
       float *acc = sc.gacc + (size_t)ev_idx * 16;
 #pragma unroll
       for (int r = 0; r < 3; ++r) {
@@ -316,7 +403,7 @@ template <int DEG, bool RS>
 ut_status launch_k(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, const uint32_t *vals,
                    const uint32_t *ranges, const TileSched &ts, cudaStream_t s) {
   const int threads = op.tile_w * op.tile_h;
-  const size_t smem = sizeof(float) * 6 * (size_t)op.kbuffer * threads + sizeof(WarpRays) * (threads / 32);
+  const size_t smem = sizeof(float) * 6 * (size_t)op.kbuffer * threads + (sizeof(WarpRays) + 96 * sizeof(float)) * (threads / 32);
   constexpr size_t kStatic = sizeof(float4) * kBatchKB * 5 + sizeof(float) * kBatchKB * 3 * (DEG + 1) * (DEG + 1) +
                              sizeof(uint32_t) * kBatchKB;
   if (smem + kStatic > 227 * 1024) return UT_ERR_UNSUPPORTED;  // the buffer does not fit one block
