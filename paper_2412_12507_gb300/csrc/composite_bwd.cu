@@ -65,12 +65,12 @@ struct __align__(16) BwdWarp {
   static constexpr int OST = NC == 48 ? 60 : (NC % 4 == 0 ? NC + 4 : NC);
   WarpRays rays;
   float4 geo[kRoundB][5];                   // stage_particle's record; o - mu or mu, list position
-  float col[kRoundB * (PP ? 4 : NC)];       // SH coefficients, or the colour (PP)
+  alignas(16) float col[kRoundB * (PP ? 4 : NC)];  // SH coefficients, or the colour (PP)
   uint32_t idx[kRoundB];
   uint32_t cidx[kSlots > kRoundB ? kSlots : kRoundB];  // particle of each column / outgoing row
   float dc[PP ? kRoundB : 1][3];            // PP: dL/dcolour of every survivor
-  uint2 A[ROWS][32];                        // basis of the pixel pairs, (hi, lo) bf16 pairs
-  union {
+  alignas(16) uint2 A[ROWS][32];                        // basis of the pixel pairs, (hi, lo) bf16 pairs
+  union alignas(16) {
     uint2 W[COLS][32];                      // SH weights of the pixel pairs, row = channel x column
     float out[(PP ? kRoundB : kSlots) * OST];
   };
@@ -158,22 +158,25 @@ __global__ void __launch_bounds__(32 * kBlockWarps, 3) k_composite_bwd(const __g
   pixel_pair<PDEG>(cam, op, x0, y0, warp, lane, q);
   const f3x2 o = q.o, d = q.d;
   uint32_t pk[2], end[2];  // the pixels with something to replay (kDead: none), and where each stops
-  float2 gr[3], Hf;  // upstream g = dL/drgb, and g . (composited colour) - dL/dalpha T_final
+  float2 gr[3], Cf[3], gAT;  // upstream dL/drgb, composited colour, dL/dalpha T_final
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
-    float u[3] = {0.f, 0.f, 0.f}, hf = 0.f;
+    float u[7] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     end[h] = 0;
     if (q.valid[h]) {
       const size_t pix = (size_t)q.py[h] * cam.W + q.px[h], plane = (size_t)cam.W * cam.H;
       end[h] = view.n_used[pix];
       u[0] = view.d_rgb[pix]; u[1] = view.d_rgb[plane + pix]; u[2] = view.d_rgb[2 * plane + pix];
-      hf = fmaf(u[0], view.rgb[pix], fmaf(u[1], view.rgb[plane + pix], u[2] * view.rgb[2 * plane + pix])) -
-           view.d_alpha[pix] * view.tfinal[pix];
+      u[3] = view.rgb[pix]; u[4] = view.rgb[plane + pix]; u[5] = view.rgb[2 * plane + pix];
+      u[6] = view.d_alpha[pix] * view.tfinal[pix];
     }
     pk[h] = end[h] > rg.x ? (uint32_t)q.px[h] | ((uint32_t)q.py[h] << 16) : kDead;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) (h ? gr[c].y : gr[c].x) = u[c];
-    (h ? Hf.y : Hf.x) = hf;
+    for (int c = 0; c < 3; ++c) {
+      (h ? gr[c].y : gr[c].x) = u[c];
+      (h ? Cf[c].y : Cf[c].x) = u[3 + c];
+    }
+    (h ? gAT.y : gAT.x) = u[6];
   }
   // no pixel of this warp blends a particle at or after `stop`
   const uint32_t stop = min(__reduce_max_sync(kFull, max(end[0], end[1])), rg.y);
@@ -227,7 +230,7 @@ __global__ void __launch_bounds__(32 * kBlockWarps, 3) k_composite_bwd(const __g
     __syncwarp();
   };
 
-  float2 T = bc(1.f), P = bc(0.f);  // transmittance, g . (running prefix of the composited colour)
+  float2 T = bc(1.f), A[3] = {bc(0.f), bc(0.f), bc(0.f)};  // transmittance, running prefix of the colour
   int cols = 0;
   uint32_t idx = list_index(vals, rg.x + lane, stop), idx1 = list_index(vals, rg.x + 32 + lane, stop);
   short4 r = list_rect(rect, view.part_off, idx, rg.x + lane, stop);
@@ -285,13 +288,18 @@ __global__ void __launch_bounds__(32 * kBlockWarps, 3) k_composite_bwd(const __g
           c1 = make_float2(h0 ? fmaxf(c1.x, 0.f) : 0.f, h1 ? fmaxf(c1.y, 0.f) : 0.f);
           c2 = make_float2(h0 ? fmaxf(c2.x, 0.f) : 0.f, h1 ? fmaxf(c2.y, 0.f) : 0.f);
           const float2 w = mul2(al, T);
-          const float2 gc = fma2(gr[0], c0, fma2(gr[1], c1, mul2(gr[2], c2)));
-          P = fma2(gc, w, P);
+          // the prefix repeats the forward's sums bit for bit, so that the colour still to come,
+          // S = C - prefix, keeps its relative accuracy down to the last particles of a ray
+          A[0] = fma2(c0, w, A[0]);
+          A[1] = fma2(c1, w, A[1]);
+          A[2] = fma2(c2, w, A[2]);
           const float2 om = make_float2(1.f - al.x, 1.f - al.y);  // >= 1 - alpha_max > 0
           const float2 inv = make_float2(__fdividef(1.f, om.x), __fdividef(1.f, om.y));
-          // dL/dalpha = sum_c g_c (c T - S_c / (1 - alpha)) + g_A T_final / (1 - alpha) with the
-          // colour still to come S = C - prefix: g . S - g_A T_final = Hf - P
-          const float2 dal = fma2(gc, T, mul2(add2(P, neg2(Hf)), inv));
+          // dL/dalpha = sum_c g_c c T + (g_A T_final - sum_c g_c S_c) / (1 - alpha)
+          const float2 gc = fma2(gr[0], c0, fma2(gr[1], c1, mul2(gr[2], c2)));
+          const float2 gs = fma2(gr[0], sub2(A[0], Cf[0]), fma2(gr[1], sub2(A[1], Cf[1]),
+                                                                  fma2(gr[2], sub2(A[2], Cf[2]), gAT)));
+          const float2 dal = fma2(gc, T, mul2(gs, inv));
           wc[0] = make_float2(c0.x > 0.f ? gr[0].x * w.x : 0.f, c0.y > 0.f ? gr[0].y * w.y : 0.f);
           wc[1] = make_float2(c1.x > 0.f ? gr[1].x * w.x : 0.f, c1.y > 0.f ? gr[1].y * w.y : 0.f);
           wc[2] = make_float2(c2.x > 0.f ? gr[2].x * w.x : 0.f, c2.y > 0.f ? gr[2].y * w.y : 0.f);

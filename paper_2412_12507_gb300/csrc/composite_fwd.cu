@@ -14,7 +14,7 @@ template <int NST>
 struct __align__(16) FwdWarp {
   WarpRays rays;
   float4 geo[kRoundF][4];       // stage_particle's record
-  float col[kRoundF * NST];     // SH coefficients, or the colour (PP)
+  alignas(16) float col[kRoundF * NST];  // SH coefficients, or the colour (PP)
   uint32_t idx[kRoundF], pos[kRoundF];  // particle, list position
 };
 
