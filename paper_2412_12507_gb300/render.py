@@ -207,20 +207,33 @@ class Renderer:
     binning: Binning | None = None
     proj: Projection | None = None
     frame: Frame | None = None
+    k_host: torch.Tensor | None = None
 
     def forward(self, scene: Scene, sync_check: bool = True):
+        """Renders one frame.  With sync_check the key count is read back and the frame rendered again
+        with a larger key capacity if it did not fit.  The count's copy is queued before the
+        compositing and waited for after the compositing is queued, so that the GPU does not idle
+        while the host reacts (an overflowing call leaves every tile's range empty: that first
+        compositing reads no keys and its black frame is overwritten)."""
         self.proj = project(scene, self.cam, self.opts, self.proj if self.proj is not None and
                             self.proj.depth.shape[0] == scene.n else None)
         while True:
             self.binning = bin_and_sort(self.proj, self.cam, self.opts, self.capacity, ws=self.ws,
                                         out=self.binning)
+            if sync_check:
+                if self.k_host is None:
+                    self.k_host = torch.empty(1, dtype=torch.int64, pin_memory=True)
+                self.k_host.copy_(self.binning.k_dev, non_blocking=True)
+                counted = torch.cuda.current_stream().record_event()
+            self.frame = composite_forward(scene, self.cam, self.opts, self.proj, self.binning, self.frame,
+                                           ws=self.fws)
             if not sync_check:
                 break
-            K = self.binning.count()
+            counted.synchronize()
+            K = int(self.k_host)
             if K <= self.binning.capacity:
                 break
             self.capacity = int(K * self.growth) + 1
-        self.frame = composite_forward(scene, self.cam, self.opts, self.proj, self.binning, self.frame, ws=self.fws)
         return self.frame
 
     def backward(self, scene: Scene, d_rgb: torch.Tensor, d_alpha: torch.Tensor):
