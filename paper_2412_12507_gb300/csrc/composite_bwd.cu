@@ -121,8 +121,9 @@ __device__ __forceinline__ void add_rows(const DevScene &sc, const float *out, i
 // threads per SM (168 registers): at 4 blocks the pair's state spills (1M rolling-shutter 1080p
 // training step 2558 us against 2520, backward of 200k particles at 640x480 890 against 780), at 5
 // far more.  Against one pixel a thread with accumulators shared by the tile's warps: that step
-// 3112 -> 2520 us, that backward 1223 -> 780 us, the 8-view step of 3M particles 58.9 -> 46.3 ms
-// (with the forward's change).
+// 3058 -> 2449 us, that backward 1143 -> 718 us, the 8-view step of 3M particles 58.9 -> 46.3 ms
+// (with the forward's change); with one branch a survivor and each reciprocal taken once:
+// 2415 -> 2269, 791 -> 669 us and 46.8 -> 42.4 ms.
 // PP (per-particle colour mode): the colour gradient dL/dc is one 3-vector per particle, summed
 // in the three spare slots of the reduce-scatter; after each round it becomes
 // dL/dbeta = dL/dc Y(dir) and the mean's gradient through the view direction.
@@ -264,82 +265,79 @@ __global__ void __launch_bounds__(32 * kBlockWarps, 3) k_composite_bwd(const __g
       const float4 g3 = S.geo[b][3], ax = S.geo[b][4];
       const uint32_t q0 = __float_as_uint(g3.z), q1 = __float_as_uint(g3.w), pos = __float_as_uint(ax.w);
       bool h0 = in_rect(pk[0], q0, q1) && pos < end[0], h1 = in_rect(pk[1], q0, q1) && pos < end[1];
-      float2 wc[3] = {bc(0.f), bc(0.f), bc(0.f)};
-      float v[16];
-#pragma unroll
-      for (int k = 0; k < 16; ++k) v[k] = 0.f;
-      if (h0 || h1) {
-        const PairEval e = eval_pair<RS>(S.geo[b][0], S.geo[b][1], S.geo[b][2], o, d);
-        h0 = h0 && e.cc.x <= g3.y * e.dd.x;
-        h1 = h1 && e.cc.y <= g3.y * e.dd.y;
-        if (h0 || h1) {
-          // a pixel that the particle does not reach has alpha 0 and takes part in no sum
-          const float2 a = make_float2(h0 ? response<GEN>(g3.x, e.cc.x, e.dd.x, op) : 0.f,
-                                       h1 ? response<GEN>(g3.x, e.cc.y, e.dd.y, op) : 0.f);
-          const float2 al = make_float2(fminf(a.x, op.alpha_max), fminf(a.y, op.alpha_max));
-          float2 c0, c1, c2;
-          if (PP) {
-            const float4 cr = reinterpret_cast<const float4 *>(S.col)[b];
-            c0 = bc(cr.x); c1 = bc(cr.y); c2 = bc(cr.z);
-          } else {
-            sh_colour2<NSH>(S.col + b * NC, q.Y, c0, c1, c2);
-          }
-          c0 = make_float2(h0 ? fmaxf(c0.x, 0.f) : 0.f, h1 ? fmaxf(c0.y, 0.f) : 0.f);
-          c1 = make_float2(h0 ? fmaxf(c1.x, 0.f) : 0.f, h1 ? fmaxf(c1.y, 0.f) : 0.f);
-          c2 = make_float2(h0 ? fmaxf(c2.x, 0.f) : 0.f, h1 ? fmaxf(c2.y, 0.f) : 0.f);
-          const float2 w = mul2(al, T);
-          // the prefix repeats the forward's sums bit for bit, so that the colour still to come,
-          // S = C - prefix, keeps its relative accuracy down to the last particles of a ray
-          A[0] = fma2(c0, w, A[0]);
-          A[1] = fma2(c1, w, A[1]);
-          A[2] = fma2(c2, w, A[2]);
-          const float2 om = make_float2(1.f - al.x, 1.f - al.y);  // >= 1 - alpha_max > 0
-          const float2 inv = make_float2(__fdividef(1.f, om.x), __fdividef(1.f, om.y));
-          // dL/dalpha = sum_c g_c c T + (g_A T_final - sum_c g_c S_c) / (1 - alpha)
-          const float2 gc = fma2(gr[0], c0, fma2(gr[1], c1, mul2(gr[2], c2)));
-          const float2 gs = fma2(gr[0], sub2(A[0], Cf[0]), fma2(gr[1], sub2(A[1], Cf[1]),
-                                                                  fma2(gr[2], sub2(A[2], Cf[2]), gAT)));
-          const float2 dal = fma2(gc, T, mul2(gs, inv));
-          wc[0] = make_float2(c0.x > 0.f ? gr[0].x * w.x : 0.f, c0.y > 0.f ? gr[0].y * w.y : 0.f);
-          wc[1] = make_float2(c1.x > 0.f ? gr[1].x * w.x : 0.f, c1.y > 0.f ? gr[1].y * w.y : 0.f);
-          wc[2] = make_float2(c2.x > 0.f ? gr[2].x * w.x : 0.f, c2.y > 0.f ? gr[2].y * w.y : 0.f);
-          T = mul2(T, om);
-          const float2 da = make_float2(!h0 || a.x > op.alpha_max ? 0.f : dal.x,
-                                        !h1 || a.y > op.alpha_max ? 0.f : dal.y);
-          v[12] = fmaf(da.x, __fdividef(a.x, g3.x), da.y * __fdividef(a.y, g3.x));
-          // 2 dL/domega^2
-          float2 dw = make_float2(-a.x * da.x, -a.y * da.y);
-          if (GEN) dw = make_float2(2.f * dresponse_w2(op, a.x, h0 ? __fdividef(e.cc.x, e.dd.x) : 0.f) * da.x,
-                                    2.f * dresponse_w2(op, a.y, h1 ? __fdividef(e.cc.y, e.dd.y) : 0.f) * da.y);
-          const float2 od = dot3x2(e.og, e.dg);
-          const float2 tau = make_float2(h0 ? -__fdividef(od.x, e.dd.x) : 0.f, h1 ? -__fdividef(od.y, e.dd.y) : 0.f);
-          const float2 vv[3] = {mul2(dw, fma2(tau, e.dg.x, e.og.x)), mul2(dw, fma2(tau, e.dg.y, e.og.y)),
-                                mul2(dw, fma2(tau, e.dg.z, e.og.z))};
-          f3x2 x;
-          if (RS) {
-            x.x = add2(o.x, bc(-ax.x));
-            x.y = add2(o.y, bc(-ax.y));
-            x.z = add2(o.z, bc(-ax.z));
-          } else {
-            x.x = bc(ax.x);
-            x.y = bc(ax.y);
-            x.z = bc(ax.z);
-          }
-          const float2 xx[3] = {fma2(tau, d.x, x.x), fma2(tau, d.y, x.y), fma2(tau, d.z, x.z)};
-#pragma unroll
-          for (int q = 0; q < 3; ++q) {
-            v[q] = vv[q].x + vv[q].y;
-#pragma unroll
-            for (int c = 0; c < 3; ++c) v[3 + 3 * q + c] = fmaf(vv[q].x, xx[c].x, vv[q].y * xx[c].y);
-          }
-        }
-      }
+      const PairEval e = eval_pair<RS>(S.geo[b][0], S.geo[b][1], S.geo[b][2], o, d);
+      h0 = h0 && e.cc.x <= g3.y * e.dd.x;
+      h1 = h1 && e.cc.y <= g3.y * e.dd.y;
       if (!__any_sync(kFull, h0 || h1)) continue;
+      // straight-line from here: a pixel that the particle does not reach has alpha 0 and takes part
+      // in no sum (its alpha, colour, dL/dalpha and tau are selected to 0, so that no infinity of its
+      // own gets in)
+      const float2 rd = make_float2(__fdividef(1.f, e.dd.x), __fdividef(1.f, e.dd.y)), w2 = mul2(e.cc, rd);
+      const float2 rho = make_float2(h0 ? response<GEN>(w2.x, op) : 0.f, h1 ? response<GEN>(w2.y, op) : 0.f);
+      const float2 a = mul2(bc(g3.x), rho);
+      const float2 al = make_float2(fminf(a.x, op.alpha_max), fminf(a.y, op.alpha_max));
+      float2 c0, c1, c2;
+      if (PP) {
+        const float4 cr = reinterpret_cast<const float4 *>(S.col)[b];
+        c0 = bc(cr.x); c1 = bc(cr.y); c2 = bc(cr.z);
+      } else {
+        sh_colour2<NSH>(S.col + b * NC, q.Y, c0, c1, c2);
+      }
+      c0 = make_float2(h0 ? fmaxf(c0.x, 0.f) : 0.f, h1 ? fmaxf(c0.y, 0.f) : 0.f);
+      c1 = make_float2(h0 ? fmaxf(c1.x, 0.f) : 0.f, h1 ? fmaxf(c1.y, 0.f) : 0.f);
+      c2 = make_float2(h0 ? fmaxf(c2.x, 0.f) : 0.f, h1 ? fmaxf(c2.y, 0.f) : 0.f);
+      const float2 w = mul2(al, T);
+      // the prefix repeats the forward's sums bit for bit, so that the colour still to come,
+      // S = C - prefix, keeps its relative accuracy down to the last particles of a ray
+      A[0] = fma2(c0, w, A[0]);
+      A[1] = fma2(c1, w, A[1]);
+      A[2] = fma2(c2, w, A[2]);
+      const float2 om = make_float2(1.f - al.x, 1.f - al.y);  // >= 1 - alpha_max > 0
+      const float2 inv = make_float2(rcp_normal(om.x), rcp_normal(om.y));
+      // dL/dalpha = sum_c g_c c T + (g_A T_final - sum_c g_c S_c) / (1 - alpha)
+      const float2 gc = fma2(gr[0], c0, fma2(gr[1], c1, mul2(gr[2], c2)));
+      const float2 gs = fma2(gr[0], sub2(A[0], Cf[0]), fma2(gr[1], sub2(A[1], Cf[1]),
+                                                              fma2(gr[2], sub2(A[2], Cf[2]), gAT)));
+      const float2 dal = fma2(gc, T, mul2(gs, inv));
+      const float2 wc[3] = {make_float2(c0.x > 0.f ? gr[0].x * w.x : 0.f, c0.y > 0.f ? gr[0].y * w.y : 0.f),
+                            make_float2(c1.x > 0.f ? gr[1].x * w.x : 0.f, c1.y > 0.f ? gr[1].y * w.y : 0.f),
+                            make_float2(c2.x > 0.f ? gr[2].x * w.x : 0.f, c2.y > 0.f ? gr[2].y * w.y : 0.f)};
+      T = mul2(T, om);
+      const float2 da = make_float2(!h0 || a.x > op.alpha_max ? 0.f : dal.x,
+                                    !h1 || a.y > op.alpha_max ? 0.f : dal.y);
+      float v[16];
+      v[12] = fmaf(da.x, rho.x, da.y * rho.y);
+      // 2 dL/domega^2
+      float2 dw = make_float2(-a.x * da.x, -a.y * da.y);
+      if (GEN) dw = make_float2(2.f * dresponse_w2(op, a.x, h0 ? w2.x : 0.f) * da.x,
+                                2.f * dresponse_w2(op, a.y, h1 ? w2.y : 0.f) * da.y);
+      const float2 od = dot3x2(e.og, e.dg);
+      const float2 tau = make_float2(h0 ? -(od.x * rd.x) : 0.f, h1 ? -(od.y * rd.y) : 0.f);
+      const float2 vv[3] = {mul2(dw, fma2(tau, e.dg.x, e.og.x)), mul2(dw, fma2(tau, e.dg.y, e.og.y)),
+                            mul2(dw, fma2(tau, e.dg.z, e.og.z))};
+      f3x2 x;
+      if (RS) {
+        x.x = add2(o.x, bc(-ax.x));
+        x.y = add2(o.y, bc(-ax.y));
+        x.z = add2(o.z, bc(-ax.z));
+      } else {
+        x.x = bc(ax.x);
+        x.y = bc(ax.y);
+        x.z = bc(ax.z);
+      }
+      const float2 xx[3] = {fma2(tau, d.x, x.x), fma2(tau, d.y, x.y), fma2(tau, d.z, x.z)};
+#pragma unroll
+      for (int q = 0; q < 3; ++q) {
+        v[q] = vv[q].x + vv[q].y;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) v[3 + 3 * q + c] = fmaf(vv[q].x, xx[c].x, vv[q].y * xx[c].y);
+      }
       const uint32_t pi = S.idx[b];
       if (PP) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) v[13 + c] = wc[c].x + wc[c].y;
       } else {
+        v[13] = v[14] = v[15] = 0.f;
         // SH weights into the next free column of W
 #pragma unroll
         for (int c = 0; c < 3; ++c) {

@@ -121,17 +121,17 @@ __global__ void __launch_bounds__(32 * kBlockWarps, fwd_blocks(DEG, RS, PP)) k_c
     if (!PP) stage_sh_warp<NC>(sc, S.idx, n, S.col, lane);
     int bl[2] = {-1, -1};  // last survivor blended by each pixel
     for (int b = 0; b < n; ++b) {
+      // no branches: nearly every survivor reaches some pixel of the warp, and straight-line code lets
+      // its loads start early; what a pixel does not blend is predicated off
       const float4 g3 = S.geo[b][3];
       const uint32_t r0 = __float_as_uint(g3.z), re = __float_as_uint(g3.w);
       bool h0 = in_rect(pk[0], r0, re), h1 = in_rect(pk[1], r0, re);
       if (STATS) n_eval += (int)h0 + (int)h1;
-      if (!(h0 || h1)) continue;
       const PairEval e = eval_pair<RS>(S.geo[b][0], S.geo[b][1], S.geo[b][2], o, d);
       h0 = h0 && e.cc.x <= g3.y * e.dd.x;
       h1 = h1 && e.cc.y <= g3.y * e.dd.y;
-      if (!(h0 || h1)) continue;
-      const float al0 = fminf(response<GEN>(g3.x, e.cc.x, e.dd.x, op), op.alpha_max);
-      const float al1 = fminf(response<GEN>(g3.x, e.cc.y, e.dd.y, op), op.alpha_max);
+      const float al0 = fminf(g3.x * response<GEN>(__fdividef(e.cc.x, e.dd.x), op), op.alpha_max);
+      const float al1 = fminf(g3.x * response<GEN>(__fdividef(e.cc.y, e.dd.y), op), op.alpha_max);
       const float Tn0 = T[0] * (1.f - al0), Tn1 = T[1] * (1.f - al1);
       if (h0 && Tn0 < op.t_min) {
         pk[0] = kDead;

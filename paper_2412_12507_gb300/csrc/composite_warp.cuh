@@ -75,11 +75,27 @@ __device__ __forceinline__ PairEval eval_pair(float4 g0, float4 g1, float4 g2, c
   return e;
 }
 
-// sigma rho(omega^2) with omega^2 = cc / dd (eval_response's arithmetic).
+// The hardware's reciprocal and power of two, one instruction each: for arguments and results known
+// to be normal numbers (subnormals count as zero).
+__device__ __forceinline__ float rcp_normal(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float exp2_normal(float x) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+// rho(omega^2) as 2^(log2(e) x exponent); alpha = sigma rho.  A pixel that passes the threshold test
+// has rho >= alpha_min / sigma >= alpha_min; where that is subnormal rho may read 0.  Other pixels'
+// values are not used.
 template <bool GEN>
-__device__ __forceinline__ float response(float sigma, float cc, float dd, const DevOpts &op) {
-  if (!GEN) return sigma * __expf(-0.5f * __fdividef(cc, dd));
-  return sigma * __expf(-op.kernel_lambda * pow_half(__fdividef(cc, dd), op.kernel_degree));
+__device__ __forceinline__ float response(float w2, const DevOpts &op) {
+  constexpr float log2e = 1.4426950408889634f;
+  if (!GEN) return exp2_normal((-0.5f * log2e) * w2);
+  return exp2_normal(log2e * (-op.kernel_lambda * pow_half(w2, op.kernel_degree)));
 }
 
 // Raw colour of a staged particle for the pixel pair (sh_colour's order of operations).
