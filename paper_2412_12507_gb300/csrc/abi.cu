@@ -539,7 +539,7 @@ ut_status composite_forward(const ut_scene *scene, const ut_camera *cam, const u
   bd.v[0].alpha = alpha;
   bd.v[0].tfinal = t_final;
   bd.v[0].n_used = n_used;
-  return launch_composite_fwd(bd, dop, rect, vals, tile_ranges, stats, workspace,
+  return launch_composite_fwd(bd, dop, rect, vals, tile_ranges, stats, workspace, false,
                               reinterpret_cast<cudaStream_t>(stream));
 }
 
@@ -626,7 +626,7 @@ ut_status render_batch(const ut_scene *scenes, int32_t n_scenes, const ut_view *
   if ((st = launch_bin(bd, depth, rect, ntiles, dop, ws + L.bin, key_capacity, nullptr, vals, ranges, k_out, s,
                        false)) != UT_OK)
     return st;
-  return launch_composite_fwd(bd, dop, rect, vals, ranges, nullptr, ws + L.sched, s);
+  return launch_composite_fwd(bd, dop, rect, vals, ranges, nullptr, ws + L.sched, true, s);
 }
 
 size_t ut_batch_backward_workspace_size(const ut_scene *scenes, int32_t n_scenes, const ut_view *views,

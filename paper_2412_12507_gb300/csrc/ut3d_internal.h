@@ -62,9 +62,11 @@ ut_status launch_bin(const BatchDesc &bd, const float *depth, const int16_t *rec
                      int64_t *k_out, cudaStream_t stream, bool short_sort);
 
 // Compositing of every global tile of the batch into the views' outputs; sched: scratch of
-// tile_sched_bytes(total tiles) for the tile order.
+// tile_sched_bytes(total tiles) for the tile order.  fixed_sequence: the same launches for every
+// tile count (a captured batch can then be updated in place).
 ut_status launch_composite_fwd(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, const uint32_t *vals,
-                               const uint32_t *ranges, unsigned long long *stats, void *sched, cudaStream_t stream);
+                               const uint32_t *ranges, unsigned long long *stats, void *sched, bool fixed_sequence,
+                               cudaStream_t stream);
 
 // Backward of the batch into the scenes' gradient outputs (accumulators cleared here).
 size_t backward_workspace_bytes(int n, bool kbuffer);  // accumulators, and the k-buffer record table
