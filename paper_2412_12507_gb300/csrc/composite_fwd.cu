@@ -323,7 +323,9 @@ __global__ void __launch_bounds__(512, 1) k_composite_fwd_kbuffer(const __grid_c
 // result depends on it): a tile's pixels saturate after roughly a fixed optical depth of
 // particles that cover the whole tile, so the estimate is the list position where
 // sum -ln(1 - 0.3 sigma) over particles whose rect contains the tile's pixels reaches
-// kFwdDepth, or the end of the first kFwdCap entries.  Every tile gets work >= 1 so that
+// kFwdDepth, or the end of the first kFwdCap entries.  Every second entry stands for two: the
+// kernel is bound by its gathers (two random L2 sectors an entry, 30 us of a 1043 us frame), and half of them order the
+// tiles as well.  Every tile gets work >= 1 so that
 // every tile, even an empty one, is scheduled (its pixels must still be written).
 constexpr int kFwdCap = 512;
 constexpr float kFwdDepth = 40.f;
@@ -342,18 +344,18 @@ __global__ void k_fwd_predict(const __grid_constant__ BatchDesc bd, DevOpts op, 
   uint32_t pred = end - rg.x;
   float tau = 0.f;
   bool found = false;
-  for (uint32_t base = rg.x; base < end && !found; base += 128) {
+  for (uint32_t base = rg.x; base < end && !found; base += 256) {
     float c[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {  // four chunks of 32 entries in flight per step
-      const uint32_t k = base + 32 * j + lane;
+      const uint32_t k = base + 64 * j + 2 * lane;
       c[j] = 0.f;
       if (k < end) {
         const uint32_t idx = vals[k];
         const short4 r = rect[view.part_off + idx];
         if (r.x <= x0 && r.y <= y0 && r.z >= x1 && r.w >= y1) {
           const float sg = 1.f / (1.f + __expf(-logits[idx]));
-          c[j] = -__logf(1.f - fminf(0.3f * sg, 0.99f));
+          c[j] = -2.f * __logf(1.f - fminf(0.3f * sg, 0.99f));
         }
       }
     }
@@ -367,7 +369,7 @@ __global__ void k_fwd_predict(const __grid_constant__ BatchDesc bd, DevOpts op, 
       }
       const unsigned hit = __ballot_sync(0xffffffffu, !found && tau + incl >= kFwdDepth);
       if (hit) {
-        pred = base + 32 * j + (__ffs(hit) - 1) + 1 - rg.x;
+        pred = min(base + 64 * j + 2 * __ffs(hit), end) - rg.x;
         found = true;
       }
       tau += __shfl_sync(0xffffffffu, incl, 31);
