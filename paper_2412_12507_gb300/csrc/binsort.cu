@@ -492,15 +492,32 @@ __global__ void __launch_bounds__(kThreads) k_depth_init(int n, const float *__r
   if (threadIdx.x == 0 && tot) atomicAdd(reinterpret_cast<unsigned long long *>(ksum), (unsigned long long)tot);
 }
 
-// Depth order -> number of tile columns each particle covers (0 if culled).
-__global__ void k_gather_widths(int n, const uint32_t *__restrict__ order, const uint32_t *__restrict__ ntiles,
-                                const short4 *__restrict__ rect, int tile_w, uint32_t *__restrict__ cnt) {
+// A particle's first column key from its rectangle: (tile rows covered << 16) | global tile column,
+// or with PACK global tile column | first tile row << 14 | (rows - 1) << 23 (the sort uses the
+// column bits only; the rest rides along for the row stage).  Its columns' keys follow by + 1.
+template <bool PACK>
+__device__ __forceinline__ uint32_t column_key(short4 r, int col_off, int tile_w, int tile_h) {
+  const uint32_t h = (uint32_t)(r.w / tile_h - r.y / tile_h + 1), col = (uint32_t)(col_off + r.x / tile_w);
+  return PACK ? (col | ((uint32_t)(r.y / tile_h) << 14) | ((h - 1u) << 23)) : ((h << 16) | col);
+}
+
+// Depth order -> number of tile columns each particle covers (0 if culled) and its first column
+// key.  The rectangle is the one random access per particle of the stage: a key other than the
+// culled ones' is a live particle's, and the culled ones come last in index order, so that their
+// ntiles (a live depth may have the culled ones' bits) are read nearly in sequence; the emission
+// reads the column key from here.
+template <bool PACK>
+__global__ void k_gather_widths(const __grid_constant__ BatchDesc bd, int n, const uint32_t *__restrict__ keys,
+                                const uint32_t *__restrict__ order, const uint32_t *__restrict__ ntiles,
+                                const short4 *__restrict__ rect, int tile_w, int tile_h, uint32_t *__restrict__ cnt,
+                                uint32_t *__restrict__ ckey) {
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
     const uint32_t g = order[j];
     uint32_t w = 0;
-    if (ntiles[g]) {
+    if (keys[j] != 0xffffffffu || ntiles[g]) {
       const short4 r = rect[g];
       w = (uint32_t)(r.z / tile_w - r.x / tile_w + 1);
+      ckey[j] = column_key<PACK>(r, bd.v[view_of_particle(bd, (int)g)].col_off, tile_w, tile_h);
     }
     cnt[j] = w;
   }
@@ -522,8 +539,8 @@ inline size_t small_sort_smem() { return sizeof(uint32_t) * (2 * (size_t)kSmallS
 
 __global__ void __launch_bounds__(kSmallThreads, 1)
     k_depth_small(int n, const float *__restrict__ depth, const uint32_t *__restrict__ ntiles,
-                  const short4 *__restrict__ rect, int tile_w, uint32_t *__restrict__ order, uint32_t *__restrict__ widths,
-                  uint32_t *__restrict__ offs, u64 *__restrict__ total, uint2 *__restrict__ ranges, int tiles,
+                  const short4 *__restrict__ rect, int tile_w, int tile_h, int pack, uint32_t *__restrict__ order,
+                  uint32_t *__restrict__ widths, uint32_t *__restrict__ ckey, uint32_t *__restrict__ offs, u64 *__restrict__ total, uint2 *__restrict__ ranges, int tiles,
                   uint32_t *__restrict__ group, int words) {
   extern __shared__ uint32_t s_small[];
   uint32_t *s_k = s_small, *s_v = s_k + kSmallSort, *s_hist = s_v + kSmallSort;  // [kSmallWarps][256]
@@ -634,6 +651,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
       if (ntiles[v[i]]) {
         const short4 r = rect[v[i]];
         w = (uint32_t)(r.z / tile_w - r.x / tile_w + 1);
+        ckey[p] = pack ? column_key<true>(r, 0, tile_w, tile_h) : column_key<false>(r, 0, tile_w, tile_h);
       }
       widths[p] = w;
     }
@@ -667,18 +685,13 @@ __device__ __forceinline__ int run_owner(uint32_t start, uint32_t p) {
 
 // Column entries, one warp per 32 particles of the depth order.  The particles' runs are
 // consecutive in the output, so the warp writes their union [start_0, end_31) with all lanes,
-// each lane finding the run of its position.  Key = (tile rows covered << 16) | global tile
-// column, or with PACK global tile column | first tile row << 14 | (rows - 1) << 23 (the sort
-// uses the column bits only; the rest rides along for the row stage), value = flattened
-// particle index.
-template <bool PACK>
-__global__ void __launch_bounds__(kThreads) k_emit_cols(const __grid_constant__ BatchDesc bd, int n,
-                                                        const uint32_t *__restrict__ order,
+// each lane finding the run of its position.  Key = the particle's first column key (column_key)
+// plus the column's place in the run, value = flattened particle index.
+__global__ void __launch_bounds__(kThreads) k_emit_cols(int n, const uint32_t *__restrict__ order,
                                                         const uint32_t *__restrict__ offs,
                                                         const uint32_t *__restrict__ widths,
-                                                        const short4 *__restrict__ rect, Count total, int tile_w,
-                                                        int tile_h, uint32_t *__restrict__ ckeys,
-                                                        uint32_t *__restrict__ cvals) {
+                                                        const uint32_t *__restrict__ ckey, Count total,
+                                                        uint32_t *__restrict__ ckeys, uint32_t *__restrict__ cvals) {
   if (total.get() == 0) return;  // nothing to emit, or more than the capacity
   const int lane = threadIdx.x & 31;
   const int nw = (int)((gridDim.x * blockDim.x) >> 5);
@@ -691,10 +704,7 @@ __global__ void __launch_bounds__(kThreads) k_emit_cols(const __grid_constant__ 
       end = start + w;
       if (w) {
         g = order[j];
-        const short4 r = rect[g];
-        const uint32_t h = (uint32_t)(r.w / tile_h - r.y / tile_h + 1);
-        const uint32_t col = (uint32_t)(bd.v[view_of_particle(bd, (int)g)].col_off + r.x / tile_w);
-        key0 = PACK ? (col | ((uint32_t)(r.y / tile_h) << 14) | ((h - 1u) << 23)) : ((h << 16) | col);
+        key0 = ckey[j];
       }
     }
     const uint32_t S = __shfl_sync(0xffffffffu, start, 0);
@@ -1425,14 +1435,19 @@ ut_status launch_bin(const BatchDesc &bd, const float *depth, const int16_t *rec
       const size_t smem = small_sort_smem();
       if (cudaFuncSetAttribute(k_depth_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return UT_ERR_CUDA;
-      k_depth_small<<<1, kSmallThreads, smem, s>>>(n, depth, ntiles, r4, op.tile_w, b.dv[0], b.cnt, b.offs, b.total,
+      k_depth_small<<<1, kSmallThreads, smem, s>>>(n, depth, ntiles, r4, op.tile_w, op.tile_h, scatter ? 1 : 0, b.dv[0],
+                                                   b.cnt, b.dk[1], b.offs, b.total,
                                                    reinterpret_cast<uint2 *>(ranges), clear ? 0 : tiles, group, (int)gtotal);
       count_launches(1);
     } else {
       // depth keys, and K = sum of ntiles (reported even when it exceeds the capacity)
       k_depth_init<<<g, kThreads, 0, s>>>(n, depth, ntiles, b.dk[0], b.dv[0], b.total + 1, group, (int)gtotal);
       r = radix_sort(b.dk, b.dv, cn, (u64)n, 0, 32, b.spine, b.chunk, s, depth_short ? group : nullptr);
-      k_gather_widths<<<g, kThreads, 0, s>>>(n, b.dv[r], ntiles, r4, op.tile_w, b.cnt);
+      uint32_t *const ckey = b.dk[r ^ 1];  // the depth sort is done with it
+      if (scatter)
+        k_gather_widths<true><<<g, kThreads, 0, s>>>(bd, n, b.dk[r], b.dv[r], ntiles, r4, op.tile_w, op.tile_h, b.cnt, ckey);
+      else
+        k_gather_widths<false><<<g, kThreads, 0, s>>>(bd, n, b.dk[r], b.dv[r], ntiles, r4, op.tile_w, op.tile_h, b.cnt, ckey);
       count_launches(2);
       scan(b.cnt, b.offs, cn, (u64)n, b.chunk, b.total, s);
     }
@@ -1447,12 +1462,7 @@ ut_status launch_bin(const BatchDesc &bd, const float *depth, const int16_t *rec
     // 2. column entries in depth order, sorted by global tile column
     const Count cc{b.total, (u64)cap, 0, b.total + 1};  // nothing is written unless K fits
     const int eg = (int)std::min<u64>((u64)(n + kThreads - 1) / kThreads, (u64)device_sm_count() * 16);
-    if (scatter)
-      k_emit_cols<true><<<eg, kThreads, 0, s>>>(bd, n, b.dv[r], b.offs, b.cnt, r4, cc, op.tile_w, op.tile_h, ck[0],
-                                                cv[0]);
-    else
-      k_emit_cols<false><<<eg, kThreads, 0, s>>>(bd, n, b.dv[r], b.offs, b.cnt, r4, cc, op.tile_w, op.tile_h, ck[0],
-                                                 cv[0]);
+    k_emit_cols<<<eg, kThreads, 0, s>>>(n, b.dv[r], b.offs, b.cnt, b.dk[r ^ 1], cc, ck[0], cv[0]);
     count_launches(1);
     const int rc = radix_sort(ck, cv, cc, (u64)cap, 0, cbits, b.spine, b.chunk, s,
                               col_short ? group + gdepth : nullptr);
