@@ -98,11 +98,11 @@ __device__ __forceinline__ float response(float w2, const DevOpts &op) {
   return exp2_normal(log2e * (-op.kernel_lambda * pow_half(w2, op.kernel_degree)));
 }
 
-// Raw colour of a staged particle for the pixel pair (sh_colour's order of operations).
+// Raw colour of a staged particle for the pixel pair (sh_colour's order of operations; the first
+// term, fmaf(beta_0, Y_0, 1/2), is the same for every pixel and staged in beta_0's place).
 template <int NSH>
 __device__ __forceinline__ void sh_colour2(const float *shb, const float2 *Y, float2 &r0, float2 &r1, float2 &r2) {
   constexpr int NC = NSH * 3;
-  r0 = r1 = r2 = bc(0.5f);
   if constexpr (NC % 4 == 0) {
     const float4 *s4 = reinterpret_cast<const float4 *>(shb);
 #pragma unroll
@@ -112,14 +112,16 @@ __device__ __forceinline__ void sh_colour2(const float *shb, const float2 *Y, fl
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const int idx = 4 * j + e, k = idx / 3, ch = idx % 3;
-        if (ch == 0) r0 = fma2(bc(cv[e]), Y[k], r0);
-        else if (ch == 1) r1 = fma2(bc(cv[e]), Y[k], r1);
-        else r2 = fma2(bc(cv[e]), Y[k], r2);
+        float2 &r = ch == 0 ? r0 : (ch == 1 ? r1 : r2);
+        r = k == 0 ? bc(cv[e]) : fma2(bc(cv[e]), Y[k], r);
       }
     }
   } else {
+    r0 = bc(shb[0]);
+    r1 = bc(shb[1]);
+    r2 = bc(shb[2]);
 #pragma unroll
-    for (int k = 0; k < NSH; ++k) {
+    for (int k = 1; k < NSH; ++k) {
       r0 = fma2(bc(shb[3 * k]), Y[k], r0);
       r1 = fma2(bc(shb[3 * k + 1]), Y[k], r1);
       r2 = fma2(bc(shb[3 * k + 2]), Y[k], r2);
@@ -384,7 +386,8 @@ __device__ __forceinline__ short4 list_rect(const short4 *__restrict__ rect, int
 }
 
 // SH coefficients of the n particles idx[] into the warp's dst, by asynchronous copies (16 bytes
-// when the rows are 16-byte aligned, else 4); complete, and visible to the warp, on return.
+// when the rows are 16-byte aligned, else 4), with beta_0 replaced by the colour's constant term
+// (sh_colour2); complete, and visible to the warp, on return.  n is at most 32.
 template <int NC>
 __device__ __forceinline__ void stage_sh_warp(const DevScene &sc, const uint32_t *idx, int n, float *dst, int lane) {
   const uint32_t d0 = (uint32_t)__cvta_generic_to_shared(dst);
@@ -405,6 +408,13 @@ __device__ __forceinline__ void stage_sh_warp(const DevScene &sc, const uint32_t
     }
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncwarp();
+  float Y0[1];
+  sh_basis<0>(0.f, 0.f, 1.f, Y0);
+  if (lane < n) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) dst[lane * NC + c] = fmaf(dst[lane * NC + c], Y0[0], 0.5f);
+  }
   __syncwarp();
 }
 
