@@ -39,10 +39,10 @@ __device__ __forceinline__ void store_pixel(const DevView &view, const DevCam &c
 constexpr int fwd_blocks(int deg, bool rs, bool pp) { return pp ? (rs ? 6 : 8) : (deg < 2 ? 6 : 4); }
 
 // Forward compositing, two pixels a thread and 64 a warp (composite_warp.cuh).  Against one pixel a
-// thread with the block's shared staging (1M rolling-shutter 1080p, k_composite_fwd alone): 578 M
-// -> 384 M warp instructions, 616 -> 507 us; composite_forward of 200k particles at 3840x2160
-// 1010 -> 835 us; the image is bit-identical.
-
+// thread with the block's shared staging: 1M rolling-shutter 1080p, this kernel alone, 578 M -> 348 M
+// warp instructions, 616 -> 470 us (issue 58 %, FMA pipe 56 % of the cycles at 16 warps an SM: bound
+// by both); composite_forward of 200k particles at 3840x2160 977 -> 806 us; 8 views of 3M particles
+// 13.4 -> 11 ms; the image is bit-identical.
 // PP: per-particle colour mode (the colour of each staged particle is evaluated once, at its
 // view direction, while staging; pixels read it from shared memory).
 template <int DEG, bool RS, bool STATS, bool PP, bool GEN>
@@ -324,9 +324,10 @@ __global__ void __launch_bounds__(512, 1) k_composite_fwd_kbuffer(const __grid_c
 // particles that cover the whole tile, so the estimate is the list position where
 // sum -ln(1 - 0.3 sigma) over particles whose rect contains the tile's pixels reaches
 // kFwdDepth, or the end of the first kFwdCap entries.  Every second entry stands for two: the
-// kernel is bound by its gathers (two random L2 sectors an entry, 30 us of a 1043 us frame), and half of them order the
-// tiles as well.  Every tile gets work >= 1 so that
-// every tile, even an empty one, is scheduled (its pixels must still be written).
+// kernel is bound by its gathers (two random L2 sectors an entry; 30 us of a 1044 us frame of 1M
+// particles at 1080p, 1027 us with half of them), and half of them order the tiles as well.  Every
+// tile gets work >= 1 so that every tile, even an empty one, is scheduled (its pixels must still
+// be written).
 constexpr int kFwdCap = 512;
 constexpr float kFwdDepth = 40.f;
 
@@ -388,9 +389,7 @@ void fwd_launch_s(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, c
   constexpr int NST = PP ? 4 : 3 * (DEG + 1) * (DEG + 1);
   const int warps = block_warps(op);
   const size_t smem = sizeof(FwdWarp<NST>) * (size_t)warps;
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_composite_fwd<DEG, RS, STATS, PP, GEN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
+  static_assert(sizeof(FwdWarp<NST>) * kBlockWarps <= 48 * 1024, "a block's dynamic shared memory needs no opt-in");
   k_composite_fwd<DEG, RS, STATS, PP, GEN><<<bd.total_tiles * tile_blocks(op), 32 * warps, smem, s>>>(
       bd, op, reinterpret_cast<const short4 *>(rect), vals, reinterpret_cast<const uint2 *>(ranges), stats, ts);
 }
