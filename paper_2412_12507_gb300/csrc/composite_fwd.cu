@@ -31,11 +31,11 @@ __device__ __forceinline__ void store_pixel(const DevView &view, const DevCam &c
 }
 
 // Resident blocks of 128 threads per SM that the kernel is compiled for.  Bound by issue and by the
-// latency of a chunk's loads, so more warps pay until the pixels' state spills.  Measured per call:
-// degree 3 on the 1M rolling-shutter 1080p view 1172 us a frame at 4 blocks (128 registers),
-// 1203 at 5, 1290 at 6; per-particle colours (no SH basis in registers) composite_forward of 200k
-// particles at 3840x2160 932 us at 5 blocks, 876 at 6, 831 at 8, but with a rolling shutter
-// 1104 us a frame at 5, 1095 at 6, 1170 at 8; degree 0 and 1 within 2 % from 5 to 8.
+// latency of a chunk's loads, so more warps pay until the pixels' state spills.  Measured:
+// degree 3 on the 1M rolling-shutter 1080p view 1021 us a frame at 4 blocks (124 registers), 1058
+// at 5; per-particle colours (no SH basis in registers) composite_forward of 200k particles at
+// 3840x2160 830 us at 6 blocks, 810 at 7, 802 at 8, but with a rolling shutter 948 us a frame at 5,
+// 954 at 6, 1013 at 8; degree 1 536 us a frame (400k particles, 1080p) at 5, 521 at 6, 528 at 8.
 constexpr int fwd_blocks(int deg, bool rs, bool pp) { return pp ? (rs ? 6 : 8) : (deg < 2 ? 6 : 4); }
 
 // Forward compositing, two pixels a thread and 64 a warp (composite_warp.cuh).  Against one pixel a
