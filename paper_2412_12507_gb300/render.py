@@ -222,7 +222,10 @@ class Renderer:
                                         out=self.binning)
             if sync_check:
                 if self.k_host is None:
-                    self.k_host = torch.empty(1, dtype=torch.int64, pin_memory=True)
+                    # an ordinary host tensor under any of the caller's modes: one made in inference
+                    # mode could not be written outside it, one on a default device not be pinned
+                    with torch.inference_mode(False):
+                        self.k_host = torch.empty(1, dtype=torch.int64, device="cpu", pin_memory=True)
                 self.k_host.copy_(self.binning.k_dev, non_blocking=True)
                 counted = torch.cuda.current_stream().record_event()
             self.frame = composite_forward(scene, self.cam, self.opts, self.proj, self.binning, self.frame,
