@@ -272,7 +272,11 @@ __global__ void __launch_bounds__(32 * kBlockWarps, 3) k_composite_bwd(const __g
       // straight-line from here: a pixel that the particle does not reach has alpha 0 and takes part
       // in no sum (its alpha, colour, dL/dalpha and tau are selected to 0, so that no infinity of its
       // own gets in)
-      const float2 rd = make_float2(__fdividef(1.f, e.dd.x), __fdividef(1.f, e.dd.y)), w2 = mul2(e.cc, rd);
+      // 1 / |d_g|^2 is taken of 2^64 |d_g|^2, and multiplied by numerators scaled alike, where |d_g|^2
+      // is small: a scale above 1e19 makes it subnormal, and its reciprocal an infinity
+      const float2 up = make_float2(e.dd.x < 0x1p-63f ? 0x1p64f : 1.f, e.dd.y < 0x1p-63f ? 0x1p64f : 1.f);
+      const float2 du = mul2(e.dd, up), rd = make_float2(rcp_normal(du.x), rcp_normal(du.y));
+      const float2 w2 = mul2(mul2(e.cc, up), rd);
       const float2 rho = make_float2(h0 ? response<GEN>(w2.x, op) : 0.f, h1 ? response<GEN>(w2.y, op) : 0.f);
       const float2 a = mul2(bc(g3.x), rho);
       const float2 al = make_float2(fminf(a.x, op.alpha_max), fminf(a.y, op.alpha_max));
@@ -311,7 +315,7 @@ __global__ void __launch_bounds__(32 * kBlockWarps, 3) k_composite_bwd(const __g
       float2 dw = make_float2(-a.x * da.x, -a.y * da.y);
       if (GEN) dw = make_float2(2.f * dresponse_w2(op, a.x, h0 ? w2.x : 0.f) * da.x,
                                 2.f * dresponse_w2(op, a.y, h1 ? w2.y : 0.f) * da.y);
-      const float2 od = dot3x2(e.og, e.dg);
+      const float2 od = mul2(dot3x2(e.og, e.dg), up);
       const float2 tau = make_float2(h0 ? -(od.x * rd.x) : 0.f, h1 ? -(od.y * rd.y) : 0.f);
       const float2 vv[3] = {mul2(dw, fma2(tau, e.dg.x, e.og.x)), mul2(dw, fma2(tau, e.dg.y, e.og.y)),
                             mul2(dw, fma2(tau, e.dg.z, e.og.z))};
