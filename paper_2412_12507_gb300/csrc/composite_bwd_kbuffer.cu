@@ -52,6 +52,14 @@ __device__ __forceinline__ void kb_reduce_scatter16(float (&v)[16], int lane) {
   v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
+// Whether the contraction keeps the SH weights g w of a pixel with upstream gradient g to 24 bits:
+// g is 0 or of a magnitude that leaves every part of split3_bf16x2 a finite normal number for the w
+// in [alpha_min t_min, 1] met in earnest.  (An infinity leaves inf - inf in the lower parts.)
+__device__ __forceinline__ bool splits_to_24_bits(float g) {
+  const float a = fabsf(g);
+  return a == 0.f || (a >= 0x1p-60f && a <= 0x1p126f);
+}
+
 // Two floats as three bf16 pairs (x = hi + mid + lo to 24 bits).
 __device__ __forceinline__ void split3_bf16x2(float x, float y, uint32_t &hi, uint32_t &mid, uint32_t &lo) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
@@ -129,6 +137,7 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
     gAT = view.d_alpha[pix] * view.tfinal[pix];
     Cf0 = view.rgb[pix]; Cf1 = view.rgb[plane + pix]; Cf2 = view.rgb[2 * plane + pix];
   }
+  const bool split = splits_to_24_bits(g0) && splits_to_24_bits(g1) && splits_to_24_bits(g2);
   float T = 1.f, A0 = 0.f, A1 = 0.f, A2 = 0.f;  // running prefix of the composited colour
   int nbuf = 0;
   bool done = !valid;
@@ -246,11 +255,21 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
     const bool leader = has_ev && __ffs(grp) - 1 == lane;
     // SH: D[basis][column] = sum over pixels of Y g_c w, columns (group, channel), two groups at a
     // time.  A lane's column is g8 (channel g8 mod 3); its pixel pairs are split once a step and
-    // masked by the column's group.
+    // masked by the column's group.  Weights that do not split are added lane by lane and take no
+    // part in the contraction.
     __syncwarp();
 #pragma unroll
-    for (int c = 0; c < 3; ++c) s_gc[32 * c + lane] = has_ev ? ev_gc[c] : 0.f;
+    for (int c = 0; c < 3; ++c) s_gc[32 * c + lane] = has_ev && split ? ev_gc[c] : 0.f;
     __syncwarp();
+    if (has_ev && !split) {
+      float *dsh = sc.d_sh + (size_t)ev_idx * NC;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        if (ev_gc[c] == 0.f) continue;
+#pragma unroll
+        for (int k = 0; k < NSH; ++k) atomicAdd(&dsh[3 * k + c], ev_gc[c] * Y[k]);
+      }
+    }
     uint32_t B[4][3];  // pixel pairs 2 t4 + {0, 8, 16, 24}
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
