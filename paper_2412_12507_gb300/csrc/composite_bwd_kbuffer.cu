@@ -11,18 +11,19 @@
 // dL/dalpha = sum_c g_c (c_c T - S_c / (1 - alpha)) + g_A T_final / (1 - alpha).  The pair's
 // canonical ray (o_g, d_g) is recomputed from the particle's staged record while its batch is in
 // shared memory (about 70% of the blends at k = 16), else from the call's per-particle record
-// table (k_kb_records: M, M mu, mu, sigma), and its contributions (the 13 geometry partials of k_finalize's layout, and dL/dbeta for the
-// unclamped channels) go to the particle's accumulators.  The lanes of a warp blend in step (one
-// blend event per lane per staged particle, and per step of the final drain), and the events of a
-// step are grouped by particle: neighbouring pixels' buffers evolve alike, so a step's 20 or so
-// events name three or four particles.  The groups' SH gradients are contracted on the tensor
-// cores, D[basis][(group, channel)] = sum over the warp's pixels of Y g_c w, two groups at a time:
-// m16n8k16 BF16 with both operands split in three (24 bits, the six leading cross terms, FP32
-// accumulation; errors against the FP64 oracle equal to those of the FP32 shuffles it replaced:
-// SH 1.07e-6 / 1.07e-6, 7.5e-7 / 7.4e-7).  The 13 geometry partials of a group of four or more
-// lanes are summed with a reduce-scatter, those of a smaller one added lane by lane.  Bound by
-// instruction issue and the latency of two blocks an SM; SH by three reduce-scatters a group cost
-// 1750 us where this costs 1207 (100k particles, 1280x720, k = 16).
+// table (k_kb_records: M, M mu, mu, sigma), and its contributions (the 13 geometry partials of
+// k_finalize's layout, and dL/dbeta for the unclamped channels) go to the particle's accumulators.
+// The lanes of a warp blend in step (one blend event per lane per staged particle, and per step of
+// the final drain), and the events of a step are grouped by particle: neighbouring pixels' buffers
+// evolve alike, so a step's 20 or so events name three or four particles.  A group of four or more
+// lanes is summed with reduce-scatters over the warp, a smaller one added lane by lane; at degree 3,
+// once the tiles fill the chip, the SH gradients of all groups are contracted on the tensor cores
+// instead (launch_kbuffer), D[basis][(group, channel)] = sum over the warp's pixels of Y g_c w, two
+// groups at a time: m16n8k16 BF16 with both operands split in three (24 bits, the six leading cross
+// terms, FP32 accumulation; errors against the FP64 oracle equal to those of the FP32 sums:
+// SH 1.07e-6 / 1.07e-6, 7.5e-7 / 7.4e-7).  Bound by instruction issue and the latency of two blocks
+// an SM.  Gradients with the forward of 100k particles, 1280x720, k = 16, degree 3: 2433 us with
+// lane-by-lane and shuffle sums, 1778 now.
 // (A window of per-list-position accumulators in shared memory was measured 5x slower: the lanes
 // of a warp blend the same particle at nearly the same time, and shared-memory atomics on one
 // address serialise, while the L2's reductions absorb them.)
@@ -97,7 +98,7 @@ __global__ void k_kb_records(const DevScene sc) {
   }
 }
 
-template <int DEG, bool RS>
+template <int DEG, bool RS, bool CONTRACT>
 __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_constant__ BatchDesc bd, DevOpts op,
                                                                const short4 *__restrict__ rect,
                                                                const uint32_t *__restrict__ vals,
@@ -108,7 +109,7 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
   __shared__ float4 s_aux[kBatchKB];
   __shared__ __align__(16) float s_sh[kBatchKB * NC];
   __shared__ uint32_t s_idx[kBatchKB];
-  extern __shared__ __align__(16) float s_kb[];  // [6][k][threads]: tau, alpha, r, g, b, list position; [warps] rays; [warps][3][32]
+  extern __shared__ __align__(16) float s_kb[];  // [6][k][threads]: tau, alpha, r, g, b, list position; [warps] rays; CONTRACT: [warps][3][32]
 
   const int tile = (int)(ts.order ? ts.order[blockIdx.x] : blockIdx.x);
   const DevView &view = bd.v[view_of_tile(bd, tile)];
@@ -219,100 +220,92 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
     has_ev = true;
   };
 
-  // adds this step's blend events to the particles' accumulators; every lane of the warp calls it
   const int lane = threadIdx.x & 31;
   WarpRays &rays = reinterpret_cast<WarpRays *>(s_kb + 6 * K * nt)[threadIdx.x >> 5];
   warp_rays1(op, px, py, o, d, valid, lane, &rays);
   const int g8 = lane >> 2, t4 = lane & 3;
-  float *s_gc = s_kb + 6 * K * nt + (sizeof(WarpRays) / 4) * (nt / 32) + 96 * (threadIdx.x >> 5);  // [3][32]
-  // A operand of emit's contraction (basis functions x the warp's 32 pixels), fixed for the tile:
-  // fragment r of k-step ks holds basis g8 (+8 for odd r) at pixels 16 ks + 2 t4 + {0, 1} (+8 for r >= 2)
+  float *s_gc = s_kb + 6 * K * nt + (sizeof(WarpRays) / 4) * (nt / 32) + 96 * (threadIdx.x >> 5);  // CONTRACT: [3][32]
+  // A operand of the contraction (basis functions x the warp's 32 pixels), fixed for the tile: fragment
+  // r of k-step ks holds basis g8 (+8 for odd r) at pixels 16 ks + 2 t4 + {0, 1} (+8 for r >= 2)
   uint32_t A[2][3][4];  // [k-step][hi, mid, lo][fragment]
+  if constexpr (CONTRACT) {
 #pragma unroll
-  for (int ks = 0; ks < 2; ++ks)
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int p = 16 * ks + 2 * t4 + (r >= 2 ? 8 : 0), kk = g8 + (r & 1 ? 8 : 0);
-      float y0 = 0.f, y1 = 0.f;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        constexpr int n = NSH;
-        const int src = k + (r & 1 ? 8 : 0);
-        if (src >= n) continue;
-        const float u0 = __shfl_sync(kFull, Y[src < n ? src : 0], p), u1 = __shfl_sync(kFull, Y[src < n ? src : 0], p + 1);
-        if (kk == src) {
-          y0 = u0;
-          y1 = u1;
-        }
-      }
-      split3_bf16x2(y0, y1, A[ks][0][r], A[ks][1][r], A[ks][2][r]);
-    }
-
-  auto emit = [&]() {
-    const unsigned act = __ballot_sync(kFull, has_ev);
-    if (!act) return;
-    const unsigned grp = __match_any_sync(kFull, has_ev ? ev_idx : 0xffffffffu);
-    const bool leader = has_ev && __ffs(grp) - 1 == lane;
-    // SH: D[basis][column] = sum over pixels of Y g_c w, columns (group, channel), two groups at a
-    // time.  A lane's column is g8 (channel g8 mod 3); its pixel pairs are split once a step and
-    // masked by the column's group.  Weights that do not split are added lane by lane and take no
-    // part in the contraction.
-    __syncwarp();
-#pragma unroll
-    for (int c = 0; c < 3; ++c) s_gc[32 * c + lane] = has_ev && split ? ev_gc[c] : 0.f;
-    __syncwarp();
-    if (has_ev && !split) {
-      float *dsh = sc.d_sh + (size_t)ev_idx * NC;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        if (ev_gc[c] == 0.f) continue;
-#pragma unroll
-        for (int k = 0; k < NSH; ++k) atomicAdd(&dsh[3 * k + c], ev_gc[c] * Y[k]);
-      }
-    }
-    uint32_t B[4][3];  // pixel pairs 2 t4 + {0, 8, 16, 24}
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float2 w = *reinterpret_cast<const float2 *>(s_gc + 32 * (g8 % 3) + 8 * q + 2 * t4);
-      split3_bf16x2(w.x, w.y, B[q][0], B[q][1], B[q][2]);
-    }
-    unsigned rem = __ballot_sync(kFull, leader);
-    const unsigned big0 = __ballot_sync(kFull, leader && __popc(grp) >= 4);
-    while (rem) {
-      const int la = __ffs(rem) - 1;
-      rem &= rem - 1;
-      const int lb = rem ? __ffs(rem) - 1 : -1;
-      rem &= rem - 1;
-      const unsigned ga = __shfl_sync(kFull, grp, la), gb = lb >= 0 ? __shfl_sync(kFull, grp, lb) : 0u;
-      const uint32_t ia = __shfl_sync(kFull, ev_idx, la), ib = __shfl_sync(kFull, ev_idx, lb >= 0 ? lb : la);
-      const unsigned cm = (g8 < 3 ? ga : (g8 < 6 ? gb : 0u)) >> (2 * t4);
-      float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int ks = 0; ks < 2; ++ks) {
-        uint32_t b[2][3];
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-          const unsigned two = cm >> (16 * ks + 8 * j);
-          const uint32_t msk = (two & 1u ? 0xffffu : 0u) | (two & 2u ? 0xffff0000u : 0u);
-#pragma unroll
-          for (int q = 0; q < 3; ++q) b[j][q] = B[2 * ks + j][q] & msk;
-        }
-        kb_mma(acc, A[ks][0], b[0][2], b[1][2]);  // smallest terms first
-        kb_mma(acc, A[ks][2], b[0][0], b[1][0]);
-        kb_mma(acc, A[ks][1], b[0][1], b[1][1]);
-        kb_mma(acc, A[ks][0], b[0][1], b[1][1]);
-        kb_mma(acc, A[ks][1], b[0][0], b[1][0]);
-        kb_mma(acc, A[ks][0], b[0][0], b[1][0]);
-      }
+    for (int ks = 0; ks < 2; ++ks)
 #pragma unroll
       for (int r = 0; r < 4; ++r) {
-        const int k = g8 + (r >= 2 ? 8 : 0), col = 2 * t4 + (r & 1);
-        if (k < NSH && col < (lb >= 0 ? 6 : 3) && acc[r] != 0.f)
-          atomicAdd(&sc.d_sh[(size_t)(col < 3 ? ia : ib) * NC + 3 * k + (col < 3 ? col : col - 3)], acc[r]);
+        const int p = 16 * ks + 2 * t4 + (r >= 2 ? 8 : 0), kk = g8 + (r & 1 ? 8 : 0);
+        float y0 = 0.f, y1 = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int src = k + (r & 1 ? 8 : 0);
+          if (src >= NSH) continue;
+          const float y = Y[src < NSH ? src : 0], u0 = __shfl_sync(kFull, y, p), u1 = __shfl_sync(kFull, y, p + 1);
+          if (kk == src) {
+            y0 = u0;
+            y1 = u1;
+          }
+        }
+        split3_bf16x2(y0, y1, A[ks][0][r], A[ks][1][r], A[ks][2][r]);
+      }
+  }
+
+  // adds this step's blend events to the particles' accumulators; every lane of the warp calls it
+  auto emit = [&]() {
+    if (!__any_sync(kFull, has_ev)) return;
+    const unsigned grp = __match_any_sync(kFull, has_ev ? ev_idx : 0xffffffffu);
+    const bool many = __popc(grp) >= 4, leader = has_ev && __ffs(grp) - 1 == lane;
+    unsigned big = __ballot_sync(kFull, leader && many);
+    if constexpr (CONTRACT) {
+      // D[basis][column] = sum over pixels of Y g_c w, columns (group, channel), two groups at a time.
+      // A lane's column is g8 (channel g8 mod 3); its pixel pairs are split once a step and masked by
+      // the column's group.  Weights that do not split take no part.
+      unsigned rem = __ballot_sync(kFull, leader);
+      __syncwarp();
+#pragma unroll
+      for (int c = 0; c < 3; ++c) s_gc[32 * c + lane] = has_ev && split ? ev_gc[c] : 0.f;
+      __syncwarp();
+      uint32_t B[4][3];  // pixel pairs 2 t4 + {0, 8, 16, 24}
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float2 w = *reinterpret_cast<const float2 *>(s_gc + 32 * (g8 % 3) + 8 * q + 2 * t4);
+        split3_bf16x2(w.x, w.y, B[q][0], B[q][1], B[q][2]);
+      }
+      while (rem) {
+        const int la = __ffs(rem) - 1;
+        rem &= rem - 1;
+        const int lb = rem ? __ffs(rem) - 1 : -1;
+        rem &= rem - 1;
+        const unsigned ga = __shfl_sync(kFull, grp, la), gb = lb >= 0 ? __shfl_sync(kFull, grp, lb) : 0u;
+        const uint32_t ia = __shfl_sync(kFull, ev_idx, la), ib = __shfl_sync(kFull, ev_idx, lb >= 0 ? lb : la);
+        const unsigned cm = (g8 < 3 ? ga : (g8 < 6 ? gb : 0u)) >> (2 * t4);
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int ks = 0; ks < 2; ++ks) {
+          uint32_t b[2][3];
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const unsigned two = cm >> (16 * ks + 8 * j);
+            const uint32_t msk = (two & 1u ? 0xffffu : 0u) | (two & 2u ? 0xffff0000u : 0u);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) b[j][q] = B[2 * ks + j][q] & msk;
+          }
+          kb_mma(acc, A[ks][0], b[0][2], b[1][2]);  // smallest terms first
+          kb_mma(acc, A[ks][2], b[0][0], b[1][0]);
+          kb_mma(acc, A[ks][1], b[0][1], b[1][1]);
+          kb_mma(acc, A[ks][0], b[0][1], b[1][1]);
+          kb_mma(acc, A[ks][1], b[0][0], b[1][0]);
+          kb_mma(acc, A[ks][0], b[0][0], b[1][0]);
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const int k = g8 + (r >= 2 ? 8 : 0), col = 2 * t4 + (r & 1);
+          if (k < NSH && col < (lb >= 0 ? 6 : 3) && acc[r] != 0.f)
+            atomicAdd(&sc.d_sh[(size_t)(col < 3 ? ia : ib) * NC + 3 * k + (col < 3 ? col : col - 3)], acc[r]);
+        }
       }
     }
-    // geometry: groups of four or more lanes by reduce-scatter, smaller ones lane by lane
-    unsigned big = big0;
+    // groups of four or more lanes by reduce-scatters of 16 values: the 13 geometry partials (with
+    // the SH gradients of degree 0 in the spare slots), and the SH gradients in rows of 16
     const int vi = lane >> 1;
     while (big) {
       const int l = __ffs(big) - 1;
@@ -326,13 +319,27 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
         v[r] = in ? ev_v[r] : 0.f;
 #pragma unroll
         for (int c = 0; c < 3; ++c) v[3 + 3 * r + c] = in ? ev_v[r] * ev_x[c] : 0.f;
+        v[13 + r] = NSH == 1 && in ? ev_gc[r] * Y[0] : 0.f;
       }
       v[12] = in ? ev_dsig : 0.f;
-      v[13] = v[14] = v[15] = 0.f;
       kb_reduce_scatter16(v, lane);
-      if (!(lane & 1) && vi < 13) atomicAdd(&sc.gacc[(size_t)p0 * 16 + vi], v[0]);
+      if (!(lane & 1)) {
+        if (vi < 13) atomicAdd(&sc.gacc[(size_t)p0 * 16 + vi], v[0]);
+        else if (NSH == 1 && v[0] != 0.f) atomicAdd(&sc.d_sh[(size_t)p0 * 3 + vi - 13], v[0]);
+      }
+      if constexpr (!CONTRACT && NSH > 1) {
+#pragma unroll
+        for (int j0 = 0; j0 < NC; j0 += 16) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            v[j] = in && j0 + j < NC ? ev_gc[(j0 + j) % 3] * Y[j0 + j < NC ? (j0 + j) / 3 : 0] : 0.f;
+          kb_reduce_scatter16(v, lane);
+          if (!(lane & 1) && j0 + vi < NC && v[0] != 0.f) atomicAdd(&sc.d_sh[(size_t)p0 * NC + j0 + vi], v[0]);
+        }
+      }
     }
-    if (has_ev && __popc(grp) < 4) {
+    // smaller ones lane by lane
+    if (has_ev && !many) {
       float *acc = sc.gacc + (size_t)ev_idx * 16;
 #pragma unroll
       for (int r = 0; r < 3; ++r) {
@@ -341,6 +348,15 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
         for (int c = 0; c < 3; ++c) atomicAdd(&acc[3 + 3 * r + c], ev_v[r] * ev_x[c]);
       }
       atomicAdd(&acc[12], ev_dsig);
+    }
+    if (has_ev && (CONTRACT ? !split : !many)) {
+      float *dsh = sc.d_sh + (size_t)ev_idx * NC;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        if (ev_gc[c] == 0.f) continue;
+#pragma unroll
+        for (int k = 0; k < NSH; ++k) atomicAdd(&dsh[3 * k + c], ev_gc[c] * Y[k]);
+      }
     }
     has_ev = false;
   };
@@ -418,23 +434,44 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
   }
 }
 
-template <int DEG, bool RS>
+template <int DEG, bool RS, bool CONTRACT>
 ut_status launch_k(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, const uint32_t *vals,
                    const uint32_t *ranges, const TileSched &ts, cudaStream_t s) {
   const int threads = op.tile_w * op.tile_h;
-  const size_t smem = sizeof(float) * 6 * (size_t)op.kbuffer * threads + (sizeof(WarpRays) + 96 * sizeof(float)) * (threads / 32);
+  const size_t smem = sizeof(float) * 6 * (size_t)op.kbuffer * threads +
+                      (sizeof(WarpRays) + (CONTRACT ? 96 * sizeof(float) : 0)) * (threads / 32);
   constexpr size_t kStatic = sizeof(float4) * kBatchKB * 5 + sizeof(float) * kBatchKB * 3 * (DEG + 1) * (DEG + 1) +
                              sizeof(uint32_t) * kBatchKB;
   if (smem + kStatic > 227 * 1024) return UT_ERR_UNSUPPORTED;  // the buffer does not fit one block
-  if (cudaFuncSetAttribute(k_composite_bwd_kbuffer<DEG, RS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem) != cudaSuccess ||
-      cudaFuncSetAttribute(k_composite_bwd_kbuffer<DEG, RS>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                           cudaSharedmemCarveoutMaxShared) != cudaSuccess)
+  const auto kernel = k_composite_bwd_kbuffer<DEG, RS, CONTRACT>;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
+      cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) !=
+          cudaSuccess)
     return UT_ERR_CUDA;
-  k_composite_bwd_kbuffer<DEG, RS><<<bd.total_tiles, threads, smem, s>>>(
-      bd, op, reinterpret_cast<const short4 *>(rect), vals, reinterpret_cast<const uint2 *>(ranges), ts);
+  kernel<<<bd.total_tiles, threads, smem, s>>>(bd, op, reinterpret_cast<const short4 *>(rect), vals,
+                                               reinterpret_cast<const uint2 *>(ranges), ts);
   count_launches(1);
   return UT_OK;
+}
+
+// How the SH gradients of a step's groups are summed.  On the tensor cores, small groups and all, when
+// a group has 48 of them and the tiles fill the chip: the L2's reductions, which the small groups'
+// lane-by-lane sums load with a sector a value, are then the bound (100k particles, 1280x720,
+// k = 16, forward and gradients: 2126 us with groups of four and more on the tensor cores, 1889 with
+// two and more, 1771 with all).  Otherwise in FP32, groups of four and more by reduce-scatters: one
+// of 16 values takes a third of what a group's contraction takes, and fewer values make small groups
+// cheap (gradients alone of 100k particles at 640x480, k = 16: degree 0 850 us on the tensor cores
+// and 529 so, degree 1 861 and 604, degree 2 976 and 769; 2000 particles over 400x300, k = 1: 1109 and
+// 805, 1094 and 905, 1243 and 1131).  Where a few tiles leave the chip idle the contraction's chain
+// of dependent MMAs is the bound (50k faint particles at 64x64, k = 16, 8 x 8 tiles, degree 3: 3201
+// and 2029).
+template <int DEG, bool RS>
+ut_status launch_kbuffer(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, const uint32_t *vals,
+                         const uint32_t *ranges, const TileSched &ts, cudaStream_t s) {
+  if constexpr (DEG == 3) {
+    if (bd.total_tiles > device_sm_count()) return launch_k<DEG, RS, true>(bd, op, rect, vals, ranges, ts, s);
+  }
+  return launch_k<DEG, RS, false>(bd, op, rect, vals, ranges, ts, s);
 }
 
 }  // namespace
@@ -458,10 +495,10 @@ ut_status launch_composite_bwd_kbuffer(const BatchDesc &bd, const DevOpts &op, c
   else if (ut_status st = launch_walk_order(bd, op, rect, vals, ranges, sched, s); st != UT_OK) return st;
   const bool rs = any_rs(bd);
   switch (bd.s[0].deg) {
-    case 0: return rs ? launch_k<0, true>(bd, op, rect, vals, ranges, ts, s) : launch_k<0, false>(bd, op, rect, vals, ranges, ts, s);
-    case 1: return rs ? launch_k<1, true>(bd, op, rect, vals, ranges, ts, s) : launch_k<1, false>(bd, op, rect, vals, ranges, ts, s);
-    case 2: return rs ? launch_k<2, true>(bd, op, rect, vals, ranges, ts, s) : launch_k<2, false>(bd, op, rect, vals, ranges, ts, s);
-    default: return rs ? launch_k<3, true>(bd, op, rect, vals, ranges, ts, s) : launch_k<3, false>(bd, op, rect, vals, ranges, ts, s);
+    case 0: return rs ? launch_kbuffer<0, true>(bd, op, rect, vals, ranges, ts, s) : launch_kbuffer<0, false>(bd, op, rect, vals, ranges, ts, s);
+    case 1: return rs ? launch_kbuffer<1, true>(bd, op, rect, vals, ranges, ts, s) : launch_kbuffer<1, false>(bd, op, rect, vals, ranges, ts, s);
+    case 2: return rs ? launch_kbuffer<2, true>(bd, op, rect, vals, ranges, ts, s) : launch_kbuffer<2, false>(bd, op, rect, vals, ranges, ts, s);
+    default: return rs ? launch_kbuffer<3, true>(bd, op, rect, vals, ranges, ts, s) : launch_kbuffer<3, false>(bd, op, rect, vals, ranges, ts, s);
   }
 }
 
