@@ -277,7 +277,7 @@ __global__ void __launch_bounds__(32 * kBlockWarps, 3) k_composite_bwd(const __g
       const float2 up = make_float2(e.dd.x < 0x1p-63f ? 0x1p64f : 1.f, e.dd.y < 0x1p-63f ? 0x1p64f : 1.f);
       const float2 du = mul2(e.dd, up), rd = make_float2(rcp_normal(du.x), rcp_normal(du.y));
       const float2 w2 = mul2(mul2(e.cc, up), rd);
-      const float2 rho = make_float2(h0 ? response<GEN>(w2.x, op) : 0.f, h1 ? response<GEN>(w2.y, op) : 0.f);
+      const float2 rho = sel2(h0, h1, response2<GEN>(w2, op), bc(0.f));
       const float2 a = mul2(bc(g3.x), rho);
       const float2 al = make_float2(fminf(a.x, op.alpha_max), fminf(a.y, op.alpha_max));
       float2 c0, c1, c2;
@@ -313,8 +313,7 @@ __global__ void __launch_bounds__(32 * kBlockWarps, 3) k_composite_bwd(const __g
       v[12] = fmaf(da.x, rho.x, da.y * rho.y);
       // 2 dL/domega^2
       float2 dw = make_float2(-a.x * da.x, -a.y * da.y);
-      if (GEN) dw = make_float2(2.f * dresponse_w2(op, a.x, h0 ? w2.x : 0.f) * da.x,
-                                2.f * dresponse_w2(op, a.y, h1 ? w2.y : 0.f) * da.y);
+      if (GEN) dw = mul2(mul2(bc(2.f), dresponse2(op, a, sel2(h0, h1, w2, bc(0.f)))), da);
       const float2 od = mul2(dot3x2(e.og, e.dg), up);
       const float2 tau = make_float2(h0 ? -(od.x * rd.x) : 0.f, h1 ? -(od.y * rd.y) : 0.f);
       const float2 vv[3] = {mul2(dw, fma2(tau, e.dg.x, e.og.x)), mul2(dw, fma2(tau, e.dg.y, e.og.y)),

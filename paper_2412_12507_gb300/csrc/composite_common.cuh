@@ -169,11 +169,6 @@ __device__ __forceinline__ bool eval_response(const float4 *g, int px, int py, f
   return true;
 }
 
-// d rho / d omega^2 times sigma for the degree-n kernel, from a = sigma rho at omega^2 = w2.
-__device__ __forceinline__ float dresponse_w2(const DevOpts &op, float a, float w2) {
-  return -op.kernel_lambda * 0.5f * (float)op.kernel_degree * pow_half(w2, op.kernel_degree - 2) * a;
-}
-
 // Per-particle colour mode: unit view direction of a particle, from the camera centre at the
 // mean's shutter time (the rolling-shutter fixed point; t = 0 for a global shutter) to the
 // mean, and 1 / the distance.

@@ -130,8 +130,8 @@ __global__ void __launch_bounds__(32 * kBlockWarps, fwd_blocks(DEG, RS, PP)) k_c
       const PairEval e = eval_pair<RS>(S.geo[b][0], S.geo[b][1], S.geo[b][2], o, d);
       h0 = h0 && e.cc.x <= g3.y * e.dd.x;
       h1 = h1 && e.cc.y <= g3.y * e.dd.y;
-      const float al0 = fminf(g3.x * response<GEN>(__fdividef(e.cc.x, e.dd.x), op), op.alpha_max);
-      const float al1 = fminf(g3.x * response<GEN>(__fdividef(e.cc.y, e.dd.y), op), op.alpha_max);
+      const float2 rho = response2<GEN>(make_float2(__fdividef(e.cc.x, e.dd.x), __fdividef(e.cc.y, e.dd.y)), op);
+      const float al0 = fminf(g3.x * rho.x, op.alpha_max), al1 = fminf(g3.x * rho.y, op.alpha_max);
       const float Tn0 = T[0] * (1.f - al0), Tn1 = T[1] * (1.f - al1);
       if (h0 && Tn0 < op.t_min) {
         pk[0] = kDead;
