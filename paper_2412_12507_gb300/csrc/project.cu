@@ -27,7 +27,7 @@ __device__ __forceinline__ bool proj_world(const DevCam &c, int rs_iters, float3
   else return project_world_t<CAM / 2, (CAM & 1) != 0>(c, rs_iters, y, uv, t);
 }
 
-// Two points at once (packed arithmetic, the same results).
+// Two points at once (packed arithmetic).
 template <int CAM>
 __device__ __forceinline__ bool proj_world2(const DevCam &c, int rs_iters, const f3x2 &y, float2 &u, float2 &v) {
   if constexpr (CAM >= 0) return project_world2<CAM / 2, (CAM & 1) != 0>(c, rs_iters, y, u, v);

@@ -248,22 +248,22 @@ __device__ __forceinline__ float3 cam_point_at(const DevCam &c, float3 y, float 
   return c.rs ? cam_point_at_t<true>(c, y, t) : cam_point_at_t<false>(c, y, t);
 }
 
-__device__ __forceinline__ float theta_d_poly(const DevCam &c, float th) {
+__host__ __device__ __forceinline__ float theta_d_poly(const DevCam &c, float th) {
   float t2 = th * th;
   return th * fmaf(t2, fmaf(t2, fmaf(t2, fmaf(t2, c.k4, c.k3), c.k2), c.k1), 1.f);
 }
 
-__device__ __forceinline__ float theta_d_prime(const DevCam &c, float th) {
+__host__ __device__ __forceinline__ float theta_d_prime(const DevCam &c, float th) {
   float t2 = th * th;
   return fmaf(t2, fmaf(t2, fmaf(t2, fmaf(t2, 9.f * c.k4, 7.f * c.k3), 5.f * c.k2), 3.f * c.k1), 1.f);
 }
 
 // Radial pinhole: r_d(r) = r (1 + k1 r^2 + k2 r^4 + k3 r^6) and its derivative.
-__device__ __forceinline__ float radial_scale(const DevCam &c, float r2) {
+__host__ __device__ __forceinline__ float radial_scale(const DevCam &c, float r2) {
   return fmaf(r2, fmaf(r2, fmaf(r2, c.k3, c.k2), c.k1), 1.f);
 }
 
-__device__ __forceinline__ float radial_prime(const DevCam &c, float r2) {
+__host__ __device__ __forceinline__ float radial_prime(const DevCam &c, float r2) {
   return fmaf(r2, fmaf(r2, fmaf(r2, 7.f * c.k3, 5.f * c.k2), 3.f * c.k1), 1.f);
 }
 
@@ -420,9 +420,10 @@ __device__ __forceinline__ PixelPlane pixel_plane(const DevCam &c, int px, int p
 // overlap; each takes exactly the steps it would take alone.  Radii with live[] false are left 0.
 // In FP32 the iteration often ends in two neighbouring values that step to each other; since both
 // then bound the bracket they do so for ever, and the value that the last of newton_iters steps
-// would leave follows from the number of steps left.
+// would leave follows from the number of steps left.  (The host form is for the test that compares
+// it with the plain loop.)
 template <int P>
-__device__ __forceinline__ void undistort(const DevCam &c, const float (&rd)[P], const bool (&live)[P],
+__host__ __device__ __forceinline__ void undistort(const DevCam &c, const float (&rd)[P], const bool (&live)[P],
                                           int newton_iters, float (&x)[P]) {
   const bool radial = c.model == UT_CAM_PINHOLE_RADIAL;
   float lo[P], hi[P], prev[P];  // prev: the iterate that a Newton step led to x from
@@ -468,7 +469,9 @@ __device__ __forceinline__ void undistort(const DevCam &c, const float (&rd)[P],
 // ---------------------------------------------------------------- two points at a time
 //
 // The pair forms of sincos_pi, rotate_axis(_fast), cam_project(_fast)_t and project_world_t: the same
-// operations in the same order for each point, with the FMAs packed.
+// operations for each point, with the FMAs packed.  (The scalar forms leave the contraction of their
+// plain products and sums to the compiler; where it chooses another one, a pair's point differs from
+// the scalar form's by that rounding.)
 __device__ __forceinline__ void sincos_pi2(float2 th, float2 &s, float2 &c) {
   const float2 k = make_float2(rintf(th.x * 0.63661977236758134f), rintf(th.y * 0.63661977236758134f));
   float2 r = fma2(neg2(k), bc(1.5707963705062866f), th);
