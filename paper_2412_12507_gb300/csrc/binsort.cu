@@ -383,8 +383,9 @@ __device__ __forceinline__ void load_radix_tile(const uint32_t *__restrict__ key
 // totals' exclusive scan, plus its digit's totals in the groups before its tile's and counts in
 // the group's tiles before it: at most nb / 16 + 15 coalesced loads a thread), which saves the two
 // scan launches (bin_and_sort of 300k particles at 1920x1080: 182 us with four launches a pass,
-// 153 with two).  1024 tiles (2M keys): 79 loads of a kilobyte row for a tile of 16 KB; beyond, they
-// would outgrow the two scans, which cost about 8 us.
+// 153 with two).  1024 tiles (2M keys): 79 loads of a kilobyte row for a tile of 16 KB, and still no
+// slower than the two scans, about 8 us (640x480, 1M particles 240 -> 206 us, 2,097,152 300 -> 290; one
+// more, with the scans, 299); beyond, the loads would outgrow them.
 constexpr uint32_t kSelfRadixTiles = 1024;
 
 template <bool SELF>
@@ -552,7 +553,10 @@ __global__ void k_gather_widths(const __grid_constant__ BD bd, int n, const uint
 // and the latency of each (about 2.5 us apiece, 30 us of a 230 us frame of 1000 particles).  The
 // keys stay in shared memory; each pass ranks them like k_radix_downsweep (warp-contiguous
 // segments, same-digit lanes by ballots), and a pass whose digit is the same for every key is
-// skipped.  It also clears the tile ranges, which the row stage fills, when they are few.
+// skipped.  It also clears the tile ranges, which the row stage fills, when they are few.  8192 keys and
+// their values are what one block holds in shared memory with its digit counts (96 KB) and sorts 8 a
+// thread: bin_and_sort at 640x480 of 4096 particles 102 us for 144 with the twelve launches, of 8192
+// 115 for 142 (8193: 141).
 constexpr int kSmallThreads = 1024;
 constexpr int kSmallWarps = kSmallThreads / 32;
 constexpr int kSmallIPT = 8;
@@ -563,8 +567,9 @@ inline size_t small_sort_smem() { return sizeof(uint32_t) * (2 * (size_t)kSmallS
 __global__ void __launch_bounds__(kSmallThreads, 1)
     k_depth_small(int n, const float *__restrict__ depth, const uint32_t *__restrict__ ntiles,
                   const short4 *__restrict__ rect, int tile_w, int tile_h, int pack, uint32_t *__restrict__ order,
-                  uint32_t *__restrict__ widths, uint32_t *__restrict__ ckey, uint32_t *__restrict__ offs, u64 *__restrict__ total, uint2 *__restrict__ ranges, int tiles,
-                  uint32_t *__restrict__ group, int words) {
+                  uint32_t *__restrict__ widths, uint32_t *__restrict__ ckey, uint32_t *__restrict__ offs,
+                  u64 *__restrict__ total, uint2 *__restrict__ ranges, int tiles, uint32_t *__restrict__ group,
+                  int words) {
   extern __shared__ uint32_t s_small[];
   uint32_t *s_k = s_small, *s_v = s_k + kSmallSort, *s_hist = s_v + kSmallSort;  // [kSmallWarps][256]
   __shared__ u64 s_warp[kSmallWarps];
@@ -1417,6 +1422,7 @@ size_t bin_workspace_bytes(int n, int64_t cap, int tiles, int cols, int max_rows
 ut_status launch_bin(const BatchDesc &bd, const float *depth, const int16_t *rect, const uint32_t *ntiles,
                      const DevOpts &op, void *ws, int64_t cap, uint64_t *keys, uint32_t *vals, uint32_t *ranges,
                      int64_t *k_out, cudaStream_t s, bool short_sort) {
+  if (short_sort && (bd.nv != 1 || bd.v[0].col_off != 0)) return UT_ERR_INVALID_ARG;
   const int n = bd.total_particles;
   const int tiles = bd.total_tiles;
   const short4 *r4 = reinterpret_cast<const short4 *>(rect);
@@ -1466,9 +1472,10 @@ ut_status launch_bin(const BatchDesc &bd, const float *depth, const int16_t *rec
       const size_t smem = small_sort_smem();
       if (cudaFuncSetAttribute(k_depth_small, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
         return UT_ERR_CUDA;
-      k_depth_small<<<1, kSmallThreads, smem, s>>>(n, depth, ntiles, r4, op.tile_w, op.tile_h, scatter ? 1 : 0, b.dv[0],
-                                                   b.cnt, b.dk[1], b.offs, b.total,
-                                                   reinterpret_cast<uint2 *>(ranges), clear ? 0 : tiles, group, (int)gtotal);
+      k_depth_small<<<1, kSmallThreads, smem, s>>>(n, depth, ntiles, r4, op.tile_w, op.tile_h, scatter ? 1 : 0,
+                                                   b.dv[0], b.cnt, b.dk[1], b.offs, b.total,
+                                                   reinterpret_cast<uint2 *>(ranges), clear ? 0 : tiles, group,
+                                                   (int)gtotal);
       count_launches(1);
     } else {
       // depth keys, and K = sum of ntiles (reported even when it exceeds the capacity)
@@ -1476,10 +1483,9 @@ ut_status launch_bin(const BatchDesc &bd, const float *depth, const int16_t *rec
       r = radix_sort(b.dk, b.dv, cn, (u64)n, 0, 32, b.spine, b.chunk, s, depth_short ? group : nullptr);
       uint32_t *const ckey = b.dk[r ^ 1];  // the depth sort is done with it
       with_desc([&](const auto &d) {
-        if (scatter)
-          k_gather_widths<true><<<g, kThreads, 0, s>>>(d, n, b.dk[r], b.dv[r], ntiles, r4, op.tile_w, op.tile_h, b.cnt, ckey);
-        else
-          k_gather_widths<false><<<g, kThreads, 0, s>>>(d, n, b.dk[r], b.dv[r], ntiles, r4, op.tile_w, op.tile_h, b.cnt, ckey);
+        const auto kern = scatter ? k_gather_widths<true, std::decay_t<decltype(d)>>
+                                  : k_gather_widths<false, std::decay_t<decltype(d)>>;
+        kern<<<g, kThreads, 0, s>>>(d, n, b.dk[r], b.dv[r], ntiles, r4, op.tile_w, op.tile_h, b.cnt, ckey);
       });
       count_launches(2);
       scan(b.cnt, b.offs, cn, (u64)n, b.chunk, b.total, s);
@@ -1514,8 +1520,8 @@ ut_status launch_bin(const BatchDesc &bd, const float *depth, const int16_t *rec
       with_desc([&](const auto &d) {
         // (with one column pass the bounds come from its digit counts)
         k_chunk_plan<<<1, 1024, 0, s>>>(d, b.colb, b.plan, dspine, cp == 1 ? 1 << cbits : 0, cc, col_short ? 1 : 0);
-        k_row_count<<<blocks, kThreads, sizeof(uint32_t) * kWarps * (max_rows + 1), s>>>(d, ckc, b.colb, b.plan, max_rows,
-                                                                                         b.tspine);
+        k_row_count<<<blocks, kThreads, sizeof(uint32_t) * kWarps * (max_rows + 1), s>>>(d, ckc, b.colb, b.plan,
+                                                                                         max_rows, b.tspine);
       });
       count_launches(2);
       const u64 tmax = plan_spine_words(max_rows, tiles, bd.total_cols);

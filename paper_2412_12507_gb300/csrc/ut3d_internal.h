@@ -54,9 +54,11 @@ size_t bin_workspace_bytes(int n, int64_t cap, int tiles, int cols, int max_rows
 ut_status bin_check_args(int32_t n, const float *depth, const int16_t *rect, const uint32_t *ntiles,
                          const ut_camera *cam, const ut_options *opt, int64_t key_capacity, const uint32_t *vals,
                          const uint32_t *tile_ranges, const int64_t *k_out, DevCam &dc, DevOpts &dop, size_t *need);
-// short_sort: a depth sort of at most 128 radix tiles skips its spine scans (fewer launches for
-// small scenes); batches pass false so that one launch sequence serves every scene size and the
-// serving loop's captured graphs stay updatable.
+// short_sort: the launches may follow the call's sizes.  The depth stage of at most 8192 particles runs
+// in one launch; radix passes over at most 1024 tiles of 2048 (particles in the depth sort, key
+// capacity in the column sort) skip their spine scans; the kernels take a descriptor of one view, so
+// it is for one view at column offset 0 only (UT_ERR_INVALID_ARG otherwise).  Batches pass false: one
+// launch sequence serves every scene size and the serving loop's captured graphs stay updatable.
 ut_status launch_bin(const BatchDesc &bd, const float *depth, const int16_t *rect, const uint32_t *ntiles,
                      const DevOpts &op, void *ws, int64_t cap, uint64_t *keys, uint32_t *vals, uint32_t *ranges,
                      int64_t *k_out, cudaStream_t stream, bool short_sort);
@@ -68,12 +70,12 @@ ut_status launch_composite_fwd(const BatchDesc &bd, const DevOpts &op, const int
                                const uint32_t *ranges, unsigned long long *stats, void *sched, bool fixed_sequence,
                                cudaStream_t stream);
 
-// Backward of the batch into the scenes' gradient outputs (accumulators cleared here).
-size_t backward_workspace_bytes(int n, bool kbuffer);  // accumulators, and the k-buffer record table
 // Orders the tiles by the forward's predicted walk, longest first, into sched.
 ut_status launch_walk_order(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, const uint32_t *vals,
                             const uint32_t *ranges, void *sched, cudaStream_t stream);
 
+// Backward of the batch into the scenes' gradient outputs (accumulators cleared here).
+size_t backward_workspace_bytes(int n, bool kbuffer);  // accumulators, and the k-buffer record table
 // Scratch of a tile schedule (forward or backward) for `tiles` tiles.
 size_t tile_sched_bytes(int tiles);
 ut_status launch_composite_bwd(const BatchDesc &bd, const DevOpts &op, const int16_t *rect, const uint32_t *vals,
