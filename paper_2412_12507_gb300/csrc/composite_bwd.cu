@@ -16,22 +16,6 @@
 namespace ut3d {
 namespace {
 
-// Reduce-scatter of 16 per-lane values over the 32 lanes: afterwards lanes 2i and 2i+1 hold
-// the warp total of value i.
-__device__ __forceinline__ void warp_reduce_scatter16(float (&v)[16], int lane) {
-#pragma unroll
-  for (int o = 16, L = 8; L >= 1; o >>= 1, L >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int j = 0; j < L; ++j) {
-      float send = up ? v[j] : v[j + L];
-      float keep = up ? v[j + L] : v[j];
-      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
-}
-
 // Two floats as bf16 pairs hi + lo (x = hi + lo to about 2^-17): the three-term products
 // hi*hi + hi*lo + lo*hi keep FP32-level accuracy on the BF16 tensor-core path.
 __device__ __forceinline__ void split_bf16x2(float x, float y, uint32_t &hi, uint32_t &lo) {
@@ -40,14 +24,6 @@ __device__ __forceinline__ void split_bf16x2(float x, float y, uint32_t &hi, uin
   __nv_bfloat162 l = __floats2bfloat162_rn(x - hf.x, y - hf.y);
   hi = *reinterpret_cast<uint32_t *>(&h);
   lo = *reinterpret_cast<uint32_t *>(&l);
-}
-
-// D += A B for one m16n8k16 BF16 tile (FP32 accumulate).
-__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
 constexpr int kSlots = 8;     // particle columns of one tensor-core flush (the MMA's N)
@@ -128,10 +104,9 @@ __device__ __forceinline__ void add_rows(const DevScene &sc, const float *out, i
 // in the three spare slots of the reduce-scatter; after each round it becomes
 // dL/dbeta = dL/dc Y(dir) and the mean's gradient through the view direction.
 template <int DEG, bool RS, bool PP, bool GEN>
-__global__ void __launch_bounds__(32 * kBlockWarps, 3) k_composite_bwd(const __grid_constant__ BatchDesc bd, DevOpts op,
-                                                          const short4 *__restrict__ rect,
-                                                          const uint32_t *__restrict__ vals,
-                                                          const uint2 *__restrict__ ranges, TileSched ts) {
+__global__ void __launch_bounds__(32 * kBlockWarps, 3)
+    k_composite_bwd(const __grid_constant__ BatchDesc bd, DevOpts op, const short4 *__restrict__ rect,
+                    const uint32_t *__restrict__ vals, const uint2 *__restrict__ ranges, TileSched ts) {
   using L = BwdWarp<DEG, PP>;
   constexpr int NSH = L::NSH;
   constexpr int NC = L::NC;

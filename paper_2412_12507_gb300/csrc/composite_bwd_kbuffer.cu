@@ -37,22 +37,6 @@ namespace {
 
 constexpr int kBatchKB = 48;  // particles staged per block step: two blocks of 256 fit an SM at k = 16
 
-// Reduce-scatter of 16 per-lane values over the 32 lanes: afterwards lanes 2i and 2i+1 hold the
-// warp total of value i.
-__device__ __forceinline__ void kb_reduce_scatter16(float (&v)[16], int lane) {
-#pragma unroll
-  for (int o = 16, L = 8; L >= 1; o >>= 1, L >>= 1) {
-    const bool up = (lane & o) != 0;
-#pragma unroll
-    for (int j = 0; j < L; ++j) {
-      const float send = up ? v[j] : v[j + L];
-      const float keep = up ? v[j + L] : v[j];
-      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
-}
-
 // Whether the contraction keeps the SH weights g w of a pixel with upstream gradient g to 24 bits:
 // g is 0 or of a magnitude that leaves every part of split3_bf16x2 a finite normal number for the w
 // in [alpha_min t_min, 1] met in earnest.  (An infinity leaves inf - inf in the lower parts.)
@@ -72,14 +56,6 @@ __device__ __forceinline__ void split3_bf16x2(float x, float y, uint32_t &hi, ui
   hi = *reinterpret_cast<const uint32_t *>(&h);
   mid = *reinterpret_cast<const uint32_t *>(&m);
   lo = *reinterpret_cast<const uint32_t *>(&l);
-}
-
-// D += A B for one m16n8k16 BF16 tile (FP32 accumulate).
-__device__ __forceinline__ void kb_mma(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
 // The record table of the scene's particles: M (row-major, 9), M mu, mu and sigma, 16 floats.
@@ -109,7 +85,8 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
   __shared__ float4 s_aux[kBatchKB];
   __shared__ __align__(16) float s_sh[kBatchKB * NC];
   __shared__ uint32_t s_idx[kBatchKB];
-  extern __shared__ __align__(16) float s_kb[];  // [6][k][threads]: tau, alpha, r, g, b, list position; [warps] rays; CONTRACT: [warps][3][32]
+  // [6][k][threads]: tau, alpha, r, g, b, list position; [warps] rays; CONTRACT: [warps][3][32]
+  extern __shared__ __align__(16) float s_kb[];
 
   const int tile = (int)(ts.order ? ts.order[blockIdx.x] : blockIdx.x);
   const DevView &view = bd.v[view_of_tile(bd, tile)];
@@ -289,12 +266,12 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
 #pragma unroll
             for (int q = 0; q < 3; ++q) b[j][q] = B[2 * ks + j][q] & msk;
           }
-          kb_mma(acc, A[ks][0], b[0][2], b[1][2]);  // smallest terms first
-          kb_mma(acc, A[ks][2], b[0][0], b[1][0]);
-          kb_mma(acc, A[ks][1], b[0][1], b[1][1]);
-          kb_mma(acc, A[ks][0], b[0][1], b[1][1]);
-          kb_mma(acc, A[ks][1], b[0][0], b[1][0]);
-          kb_mma(acc, A[ks][0], b[0][0], b[1][0]);
+          mma_bf16(acc, A[ks][0], b[0][2], b[1][2]);  // smallest terms first
+          mma_bf16(acc, A[ks][2], b[0][0], b[1][0]);
+          mma_bf16(acc, A[ks][1], b[0][1], b[1][1]);
+          mma_bf16(acc, A[ks][0], b[0][1], b[1][1]);
+          mma_bf16(acc, A[ks][1], b[0][0], b[1][0]);
+          mma_bf16(acc, A[ks][0], b[0][0], b[1][0]);
         }
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
@@ -322,7 +299,7 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
         v[13 + r] = NSH == 1 && in ? ev_gc[r] * Y[0] : 0.f;
       }
       v[12] = in ? ev_dsig : 0.f;
-      kb_reduce_scatter16(v, lane);
+      warp_reduce_scatter16(v, lane);
       if (!(lane & 1)) {
         if (vi < 13) atomicAdd(&sc.gacc[(size_t)p0 * 16 + vi], v[0]);
         else if (NSH == 1 && v[0] != 0.f) atomicAdd(&sc.d_sh[(size_t)p0 * 3 + vi - 13], v[0]);
@@ -333,7 +310,7 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
 #pragma unroll
           for (int j = 0; j < 16; ++j)
             v[j] = in && j0 + j < NC ? ev_gc[(j0 + j) % 3] * Y[j0 + j < NC ? (j0 + j) / 3 : 0] : 0.f;
-          kb_reduce_scatter16(v, lane);
+          warp_reduce_scatter16(v, lane);
           if (!(lane & 1) && j0 + vi < NC && v[0] != 0.f) atomicAdd(&sc.d_sh[(size_t)p0 * NC + j0 + vi], v[0]);
         }
       }
@@ -379,45 +356,45 @@ __global__ void __launch_bounds__(512, 1) k_composite_bwd_kbuffer(const __grid_c
     // every lane of the warp walks every particle that can reach its pixels (the emit steps are
     // warp-wide)
     for (int c0 = 0; c0 < nb; c0 += 32) {
-    unsigned m = near_mask<RS>(s_geo, c0, nb, rays, lane);
-    while (m) {
-      const int b = c0 + __ffs(m) - 1;
-      m &= m - 1;
-      float3 og, dg;
-      float dd, a;
-      bool leave = false;
-      float l_a = 0.f, l_r = 0.f, l_g = 0.f, l_b = 0.f;
-      uint32_t l_p = 0;
-      if (!done && eval_response<RS, false>(s_geo[b], px, py, o, d, og, dg, dd, a, op)) {
-        const float tau = -__fdividef(dot3(og, dg), dd);
-        const float al = fminf(a, op.alpha_max);
-        float r0, r1, r2;
-        sh_colour<NSH>(s_sh + b * NC, Y, r0, r1, r2);
-        r0 = fmaxf(r0, 0.f); r1 = fmaxf(r1, 0.f); r2 = fmaxf(r2, 0.f);
-        const uint32_t pos = start + b;
-        if (nbuf < K) {
-          kb_tau[nbuf * nt] = tau; kb_a[nbuf * nt] = al;
-          kb_r[nbuf * nt] = r0; kb_g[nbuf * nt] = r1; kb_b[nbuf * nt] = r2; kb_p[nbuf * nt] = pos;
-          ++nbuf;
-        } else {
-          // closest of the buffer and the new hit (the forward kernel's choice) leaves
-          const int bi = kb_select(kb_tau, kb_p, nt, K, tau, true);
-          leave = true;
-          if (bi < 0) {
-            l_a = al; l_r = r0; l_g = r1; l_b = r2; l_p = pos;
+      unsigned m = near_mask<RS>(s_geo, c0, nb, rays, lane);
+      while (m) {
+        const int b = c0 + __ffs(m) - 1;
+        m &= m - 1;
+        float3 og, dg;
+        float dd, a;
+        bool leave = false;
+        float l_a = 0.f, l_r = 0.f, l_g = 0.f, l_b = 0.f;
+        uint32_t l_p = 0;
+        if (!done && eval_response<RS>(s_geo[b], px, py, o, d, og, dg, dd, a)) {
+          const float tau = -__fdividef(dot3(og, dg), dd);
+          const float al = fminf(a, op.alpha_max);
+          float r0, r1, r2;
+          sh_colour<NSH>(s_sh + b * NC, Y, r0, r1, r2);
+          r0 = fmaxf(r0, 0.f); r1 = fmaxf(r1, 0.f); r2 = fmaxf(r2, 0.f);
+          const uint32_t pos = start + b;
+          if (nbuf < K) {
+            kb_tau[nbuf * nt] = tau; kb_a[nbuf * nt] = al;
+            kb_r[nbuf * nt] = r0; kb_g[nbuf * nt] = r1; kb_b[nbuf * nt] = r2; kb_p[nbuf * nt] = pos;
+            ++nbuf;
           } else {
-            l_a = kb_a[bi * nt]; l_r = kb_r[bi * nt]; l_g = kb_g[bi * nt]; l_b = kb_b[bi * nt]; l_p = kb_p[bi * nt];
-            kb_tau[bi * nt] = tau; kb_a[bi * nt] = al;
-            kb_r[bi * nt] = r0; kb_g[bi * nt] = r1; kb_b[bi * nt] = r2; kb_p[bi * nt] = pos;
+            // closest of the buffer and the new hit (the forward kernel's choice) leaves
+            const int bi = kb_select(kb_tau, kb_p, nt, K, tau, true);
+            leave = true;
+            if (bi < 0) {
+              l_a = al; l_r = r0; l_g = r1; l_b = r2; l_p = pos;
+            } else {
+              l_a = kb_a[bi * nt]; l_r = kb_r[bi * nt]; l_g = kb_g[bi * nt]; l_b = kb_b[bi * nt]; l_p = kb_p[bi * nt];
+              kb_tau[bi * nt] = tau; kb_a[bi * nt] = al;
+              kb_r[bi * nt] = r0; kb_g[bi * nt] = r1; kb_b[bi * nt] = r2; kb_p[bi * nt] = pos;
+            }
           }
         }
+        // one blend site for the warp, whichever way its lanes' hits went
+        if (leave) blend(l_a, l_r, l_g, l_b, l_p);
+        emit();
+        if (__all_sync(0xffffffffu, done)) break;
       }
-      // one blend site for the warp, whichever way its lanes' hits went
-      if (leave) blend(l_a, l_r, l_g, l_b, l_p);
-      emit();
       if (__all_sync(0xffffffffu, done)) break;
-    }
-    if (__all_sync(0xffffffffu, done)) break;
     }
   }
   // end of the list: the remaining hits in ascending (tau_max, arrival), the warp in step
@@ -494,12 +471,16 @@ ut_status launch_composite_bwd_kbuffer(const BatchDesc &bd, const DevOpts &op, c
   if (bd.total_tiles <= device_sm_count()) ts.order = nullptr;
   else if (ut_status st = launch_walk_order(bd, op, rect, vals, ranges, sched, s); st != UT_OK) return st;
   const bool rs = any_rs(bd);
+#define UT3D_KB(D)                                                           \
+  (rs ? launch_kbuffer<D, true>(bd, op, rect, vals, ranges, ts, s) \
+      : launch_kbuffer<D, false>(bd, op, rect, vals, ranges, ts, s))
   switch (bd.s[0].deg) {
-    case 0: return rs ? launch_kbuffer<0, true>(bd, op, rect, vals, ranges, ts, s) : launch_kbuffer<0, false>(bd, op, rect, vals, ranges, ts, s);
-    case 1: return rs ? launch_kbuffer<1, true>(bd, op, rect, vals, ranges, ts, s) : launch_kbuffer<1, false>(bd, op, rect, vals, ranges, ts, s);
-    case 2: return rs ? launch_kbuffer<2, true>(bd, op, rect, vals, ranges, ts, s) : launch_kbuffer<2, false>(bd, op, rect, vals, ranges, ts, s);
-    default: return rs ? launch_kbuffer<3, true>(bd, op, rect, vals, ranges, ts, s) : launch_kbuffer<3, false>(bd, op, rect, vals, ranges, ts, s);
+    case 0: return UT3D_KB(0);
+    case 1: return UT3D_KB(1);
+    case 2: return UT3D_KB(2);
+    default: return UT3D_KB(3);
   }
+#undef UT3D_KB
 }
 
 UT_DBG_READER(dbg_read_kbuffer)

@@ -130,23 +130,13 @@ __device__ __forceinline__ void sh_colour(const float *shb, const float *Y, floa
   }
 }
 
-// x^(m/2) for an integer m >= 0: repeated products (and a square root for odd m).
-__device__ __forceinline__ float pow_half(float x, int m) {
-  float p = (m & 1) ? sqrtf(x) : 1.f;
-  for (int i = 0; i < (m >> 1); ++i) p *= x;
-  return p;
-}
-
 // Response of a staged particle for the ray (o, d) of pixel (px, py).  Returns false if the
 // pixel is outside the particle's rect or sigma rho < alpha_min (tested as
-// |o_g x d_g|^2 > thr |d_g|^2).  Otherwise returns a = sigma rho(omega^2) — exp(-omega^2/2), or
-// exp(-lambda (omega^2)^(n/2)) for a kernel of degree n — and the canonical-space ray (o_g, d_g)
-// with |d_g|^2.
-// GEN: the degree-n kernel (op.kernel_degree != 2), a separate instantiation so that the
-// Gaussian path carries no test for it.
-template <bool RS, bool GEN>
+// |o_g x d_g|^2 > thr |d_g|^2).  Otherwise returns a = sigma exp(-omega^2/2) and the canonical-space
+// ray (o_g, d_g) with |d_g|^2.  (One pixel and the Gaussian kernel: the k-buffer's form.)
+template <bool RS>
 __device__ __forceinline__ bool eval_response(const float4 *g, int px, int py, float3 o, float3 d, float3 &og,
-                                              float3 &dg, float &dd, float &a, const DevOpts &op) {
+                                              float3 &dg, float &dd, float &a) {
   float4 g3 = g[3];
   int r0 = __float_as_int(g3.z), r1 = __float_as_int(g3.w);
   if (px < (r0 & 0xffff) || px > (r1 & 0xffff) || py < (r0 >> 16) || py > (r1 >> 16)) return false;
@@ -164,8 +154,7 @@ __device__ __forceinline__ bool eval_response(const float4 *g, int px, int py, f
   float cc = fmaf(c.x, c.x, fmaf(c.y, c.y, c.z * c.z));
   dd = fmaf(dg.x, dg.x, fmaf(dg.y, dg.y, dg.z * dg.z));
   if (!(cc <= g3.y * dd)) return false;
-  if (!GEN) a = g3.x * __expf(-0.5f * __fdividef(cc, dd));
-  else a = g3.x * __expf(-op.kernel_lambda * pow_half(__fdividef(cc, dd), op.kernel_degree));
+  a = g3.x * __expf(-0.5f * __fdividef(cc, dd));
   return true;
 }
 

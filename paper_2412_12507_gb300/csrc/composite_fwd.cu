@@ -46,11 +46,10 @@ constexpr int fwd_blocks(int deg, bool rs, bool pp) { return pp ? (rs ? 6 : 8) :
 // PP: per-particle colour mode (the colour of each staged particle is evaluated once, at its
 // view direction, while staging; pixels read it from shared memory).
 template <int DEG, bool RS, bool STATS, bool PP, bool GEN>
-__global__ void __launch_bounds__(32 * kBlockWarps, fwd_blocks(DEG, RS, PP)) k_composite_fwd(const __grid_constant__ BatchDesc bd, DevOpts op,
-                                                          const short4 *__restrict__ rect,
-                                                          const uint32_t *__restrict__ vals,
-                                                          const uint2 *__restrict__ ranges,
-                                                          unsigned long long *__restrict__ stats, TileSched ts) {
+__global__ void __launch_bounds__(32 * kBlockWarps, fwd_blocks(DEG, RS, PP))
+    k_composite_fwd(const __grid_constant__ BatchDesc bd, DevOpts op, const short4 *__restrict__ rect,
+                    const uint32_t *__restrict__ vals, const uint2 *__restrict__ ranges,
+                    unsigned long long *__restrict__ stats, TileSched ts) {
   constexpr int NSH = (DEG + 1) * (DEG + 1);
   constexpr int NC = NSH * 3;
   constexpr int PDEG = PP ? 0 : DEG;        // per-pixel SH basis only when colours are per pixel
@@ -265,37 +264,37 @@ __global__ void __launch_bounds__(512, 1) k_composite_fwd_kbuffer(const __grid_c
     stage_sh<NC>(sc, s_idx, nb, s_sh);
     __syncthreads();
     for (int c0 = 0; c0 < nb; c0 += 32) {
-    if (__all_sync(kFull, done)) break;
-    unsigned m = near_mask<RS>(s_geo, c0, nb, rays, lane);
-    while (m && !done) {
-      const int b = c0 + __ffs(m) - 1;
-      m &= m - 1;
-      float3 og, dg;
-      float dd, a;
-      if (!eval_response<RS, false>(s_geo[b], px, py, o, d, og, dg, dd, a, op)) continue;
-      const float tau = -__fdividef(dot3(og, dg), dd);
-      const float al = fminf(a, op.alpha_max);
-      float r0, r1, r2;
-      sh_colour<NSH>(s_sh + b * NC, Y, r0, r1, r2);
-      r0 = fmaxf(r0, 0.f); r1 = fmaxf(r1, 0.f); r2 = fmaxf(r2, 0.f);
-      const uint32_t pos = start + b;
-      if (nbuf < K) {
-        kb_tau[nbuf * nt] = tau; kb_a[nbuf * nt] = al;
-        kb_r[nbuf * nt] = r0; kb_g[nbuf * nt] = r1; kb_b[nbuf * nt] = r2; kb_p[nbuf * nt] = pos;
-        ++nbuf;
-        continue;
+      if (__all_sync(kFull, done)) break;
+      unsigned m = near_mask<RS>(s_geo, c0, nb, rays, lane);
+      while (m && !done) {
+        const int b = c0 + __ffs(m) - 1;
+        m &= m - 1;
+        float3 og, dg;
+        float dd, a;
+        if (!eval_response<RS>(s_geo[b], px, py, o, d, og, dg, dd, a)) continue;
+        const float tau = -__fdividef(dot3(og, dg), dd);
+        const float al = fminf(a, op.alpha_max);
+        float r0, r1, r2;
+        sh_colour<NSH>(s_sh + b * NC, Y, r0, r1, r2);
+        r0 = fmaxf(r0, 0.f); r1 = fmaxf(r1, 0.f); r2 = fmaxf(r2, 0.f);
+        const uint32_t pos = start + b;
+        if (nbuf < K) {
+          kb_tau[nbuf * nt] = tau; kb_a[nbuf * nt] = al;
+          kb_r[nbuf * nt] = r0; kb_g[nbuf * nt] = r1; kb_b[nbuf * nt] = r2; kb_p[nbuf * nt] = pos;
+          ++nbuf;
+          continue;
+        }
+        // closest of the buffer and the new hit (the new hit arrived last: it wins only with a
+        // strictly smaller tau_max)
+        const int bi = kb_select(kb_tau, kb_p, nt, K, tau, true);
+        if (bi < 0) {
+          blend(al, r0, r1, r2);
+        } else {
+          blend(kb_a[bi * nt], kb_r[bi * nt], kb_g[bi * nt], kb_b[bi * nt]);
+          kb_tau[bi * nt] = tau; kb_a[bi * nt] = al;
+          kb_r[bi * nt] = r0; kb_g[bi * nt] = r1; kb_b[bi * nt] = r2; kb_p[bi * nt] = pos;
+        }
       }
-      // closest of the buffer and the new hit (the new hit arrived last: it wins only with a
-      // strictly smaller tau_max)
-      const int bi = kb_select(kb_tau, kb_p, nt, K, tau, true);
-      if (bi < 0) {
-        blend(al, r0, r1, r2);
-      } else {
-        blend(kb_a[bi * nt], kb_r[bi * nt], kb_g[bi * nt], kb_b[bi * nt]);
-        kb_tau[bi * nt] = tau; kb_a[bi * nt] = al;
-        kb_r[bi * nt] = r0; kb_g[bi * nt] = r1; kb_b[bi * nt] = r2; kb_p[bi * nt] = pos;
-      }
-    }
     }
   }
   // end of the list: the remaining hits in ascending (tau_max, arrival)

@@ -1,19 +1,19 @@
 // composite_warp.cuh — the warp walk shared by the tile-order compositing forward
 // (composite_fwd.cu) and backward (composite_bwd.cu).
 //
-// A block covers an image tile (or 256 pixels of a larger one), a warp 64 of its pixels (an 8 x 8 square when the tile is made of
-// such squares), a thread two of them; the pair's arithmetic runs in packed FP32 (fma.rn.f32x2:
-// one issue slot for two FMAs, each rounded like fmaf).  Both kernels are bound by instruction
-// issue, not by memory or FP32 rate, so the layout is the one that needs the fewest warp
-// instructions per (pixel, particle): a particle's record and 48 SH coefficients are read from
-// shared memory once for 64 pixels instead of 32, and the backward's shuffle reductions run once
-// for 64 pixels.
+// A block covers an image tile (or 256 pixels of a larger one), a warp 64 of its pixels (an 8 x 8
+// square when the tile is made of such squares), a thread two of them; the pair's arithmetic runs in
+// packed FP32 (fma.rn.f32x2: one issue slot for two FMAs, each rounded like fmaf).  Both kernels are
+// bound by instruction issue, not by memory or FP32 rate, so the layout is the one that needs the
+// fewest warp instructions per (pixel, particle): a particle's record and 48 SH coefficients are
+// read from shared memory once for 64 pixels instead of 32, and the backward's shuffle reductions
+// run once for 64 pixels.
 //
 // Warps do not share staged data: each takes the tile's list 32 entries at a time, one lane per
 // entry, drops the entries that cannot reach its pixels (rect_near on the prefetched rectangles,
 // block_misses after activation), and stages only the survivors in its own shared memory.  About
-// a third to a half of the (warp, entry) pairs survive (0.34 for the multi-view 3M-particle
-// scene, 0.49 for 1M particles on one rolling-shutter 1080p view), so re-activating a particle in
+// half of the (warp, entry) pairs survive (0.43 for the multi-view 3M-particle scene, 0.54 for 1M
+// particles on one rolling-shutter 1080p view), so re-activating a particle in
 // each of a tile's warps costs less than the walk over the rest did, and no warp ever waits for
 // another one: there is no block barrier (the leading stall of a shared staging buffer).
 #pragma once
@@ -88,7 +88,7 @@ __device__ __forceinline__ float exp2_normal(float x) {
   return r;
 }
 
-// x^(m/2) of both pixels for an integer m >= 0 (pow_half's arithmetic).
+// x^(m/2) of both pixels for an integer m >= 0: repeated products (and a square root for odd m).
 __device__ __forceinline__ float2 pow_half2(float2 x, int m) {
   float2 p = (m & 1) ? make_float2(sqrtf(x.x), sqrtf(x.y)) : bc(1.f);
   for (int i = 0; i < (m >> 1); ++i) p = mul2(p, x);
@@ -143,6 +143,32 @@ __device__ __forceinline__ void sh_colour2(const float *shb, const float2 *Y, fl
       r2 = fma2(bc(shb[3 * k + 2]), Y[k], r2);
     }
   }
+}
+
+// ---------------------------------------------------------------- sums over a warp (the backwards)
+
+// Reduce-scatter of 16 per-lane values over the 32 lanes: afterwards lanes 2i and 2i+1 hold
+// the warp total of value i.
+__device__ __forceinline__ void warp_reduce_scatter16(float (&v)[16], int lane) {
+#pragma unroll
+  for (int o = 16, L = 8; L >= 1; o >>= 1, L >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int j = 0; j < L; ++j) {
+      float send = up ? v[j] : v[j + L];
+      float keep = up ? v[j + L] : v[j];
+      v[j] = keep + __shfl_xor_sync(kFull, send, o);
+    }
+  }
+  v[0] += __shfl_xor_sync(kFull, v[0], 1);
+}
+
+// D += A B for one m16n8k16 BF16 tile (FP32 accumulate).
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
 // ---------------------------------------------------------------- pixels of a warp
@@ -319,6 +345,13 @@ __device__ __forceinline__ bool rect_near(const WarpRays &w, short4 r) {
   return w.x1 >= r.x && w.x0 <= r.z && w.y1 >= r.y && w.y0 <= r.w;
 }
 
+// The approximate square root: error below 1e-6, inside the factors 1.0001 of the bounds that use it.
+__device__ __forceinline__ float sqrt_bound(float x) {
+  float r;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // True if no live pixel of the warp can pass eval_response's test |c|^2 <= thr |d_g|^2,
 // c = o_g x d_g, for the record g.  Over the warp's rays, with n = c0 / |c0| the direction of the
 // centre ray's c0 = og0 x M dc and ci = og0 x M ei,
@@ -328,15 +361,8 @@ __device__ __forceinline__ bool rect_near(const WarpRays &w, short4 r) {
 // staged M (o - mu) or M mu is shared by every pixel, so its own rounding cancels); twice that is
 // the second term of the slack.  Infinite or NaN intermediates compare false and keep the
 // particle, so only particles that eval_pair rejects for all 64 pixels are dropped: images do not
-// depend on this test.  It drops nearly everything that can be dropped (96 to 99 % of the
-// survivors reach a pixel of an 8 x 4 block), at about 3 instructions per (warp, entry).  The
-// norms come from the approximate square root (error below 1e-6, inside the factors 1.0001).
-__device__ __forceinline__ float sqrt_bound(float x) {
-  float r;
-  asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-
+// depend on this test.  It drops nearly everything that can be dropped (88 to 98 % of the survivors
+// of an 8 x 8 square reach a pixel that is still walking), at about 3 instructions per (warp, entry).
 template <bool RS>
 __device__ __forceinline__ bool block_misses(const float4 (&g)[4], const WarpRays &w) {
   const float4 g0 = g[0], g1 = g[1], g2 = g[2];
@@ -376,8 +402,8 @@ __device__ __forceinline__ unsigned near_mask(const float4 (*geo)[4], int c0, in
 #pragma unroll
     for (int q = 0; q < 4; ++q) g[q] = geo[c0 + lane][q];
     const int r0 = __float_as_int(g[3].z), r1 = __float_as_int(g[3].w);
-    near_ = rect_near(w, make_short4((short)(r0 & 0xffff), (short)(r0 >> 16), (short)(r1 & 0xffff), (short)(r1 >> 16))) &&
-            !block_misses<RS>(g, w);
+    const short4 r = make_short4((short)(r0 & 0xffff), (short)(r0 >> 16), (short)(r1 & 0xffff), (short)(r1 >> 16));
+    near_ = rect_near(w, r) && !block_misses<RS>(g, w);
   }
   return __ballot_sync(kFull, near_);
 }
