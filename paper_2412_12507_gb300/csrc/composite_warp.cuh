@@ -103,8 +103,8 @@ __device__ __forceinline__ float2 pow_half2(float2 x, int m) {
 template <bool GEN>
 __device__ __forceinline__ float2 response2(float2 w2, const DevOpts &op) {
   constexpr float log2e = 1.4426950408889634f;
-  const float2 x = GEN ? mul2(bc(log2e), mul2(bc(-op.kernel_lambda), pow_half2(w2, op.kernel_degree)))
-                       : mul2(bc(-0.5f * log2e), w2);
+  if (!GEN) return make_float2(exp2_normal((-0.5f * log2e) * w2.x), exp2_normal((-0.5f * log2e) * w2.y));
+  const float2 x = mul2(bc(log2e), mul2(bc(-op.kernel_lambda), pow_half2(w2, op.kernel_degree)));
   return make_float2(exp2_normal(x.x), exp2_normal(x.y));
 }
 
