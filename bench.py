@@ -120,6 +120,34 @@ def measured_traffic(kernel, workload_name):
     return float(rec["bytes_per_launch"])
 
 
+def link_rates(pipe, host, h2d, d2h, stream, reps=5):
+    """What the host link gave this run: the e2e step's copies alone, one direction at a time (median of
+    `reps`).  The e2e step is bound by them, and the rate differs from machine to machine."""
+    import torch
+    sc, (_, frame), out = pipe.bufs[0], pipe.graphs[0], pipe.host_out[0]
+
+    def scene_in():
+        for k, t in host.items():
+            getattr(sc, k).copy_(t.view_as(getattr(sc, k)), non_blocking=True)
+
+    def image_out():
+        out[:3].copy_(frame.rgb, non_blocking=True)
+        out[3].copy_(frame.alpha, non_blocking=True)
+
+    rates = {}
+    for name, copy, nbytes in (("h2d_gbs", scene_in, h2d), ("d2h_gbs", image_out, d2h)):
+        ms = []
+        for _ in range(reps + 1):
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record(stream)
+            copy()
+            e1.record(stream)
+            torch.cuda.synchronize()
+            ms.append(e0.elapsed_time(e1))
+        rates[name] = nbytes / statistics.median(ms[1:]) / 1e6
+    return rates
+
+
 def measure_alu_peaks(L, dev, stream, sms):
     """FP32 FMA and special-function (ex2) throughput of this GPU, from the library's probe
     kernels (ut_peak_probe: 8 independent chains per thread, 8 blocks of 256 per SM, a few ms
@@ -830,7 +858,7 @@ def run_ours(args):
 
     # end to end through the public API with host buffers: every step copies the scene in from
     # pinned host memory and the image (rgb, alpha) back out; render.FramePipeline overlaps a
-    # step's copies with the neighbouring steps' rendering (two device scene buffers, a copy
+    # step's copies with the neighbouring steps' rendering (three device scene buffers, a copy
     # stream and a read-back stream)
     host = {k: torch.as_tensor(sc_np[k]).pin_memory() for k in ("means", "log_scales", "quats", "opacity_logits", "sh")}
     pipe = render.FramePipeline(cam, op, host, int(sc_np["sh_degree"]))
@@ -851,6 +879,7 @@ def run_ours(args):
     e1.record(stream)
     barrier()
     e2e_ms = max_over_ranks(e0.elapsed_time(e1), world, dev) / e2e_steps
+    link = link_rates(pipe, host, h2d, d2h, stream)
     del pipe
 
     variants = run_variants(scene, cam, op, d_rgb, d_alpha, timed, args.steps, max(3, args.warmup))
@@ -920,7 +949,7 @@ def run_ours(args):
             "kernels": kernels, "evaluations": n_eval, "blended": n_blend, "alu_peaks": alu,
             "roofline": roofline, "cpu_baseline": cpu, "clocks": clk,
             "e2e": {"value": job_mpix_s(P, world, e2e_ms), "unit": "Mpix/s", "h2d_bytes_per_step": h2d,
-                    "d2h_bytes_per_step": d2h, "ms_per_step": e2e_ms,
+                    "d2h_bytes_per_step": d2h, "ms_per_step": e2e_ms, "link": link,
                     "overlap": "render.FramePipeline: a step's copies overlap the neighbouring steps' rendering"},
             "gpu_launches": int(launches_fwd * args.steps + launches_fb * args.steps),
             "launches_per_step": {"fwd": int(launches_fwd), "fwd_bwd": int(launches_fb)},
