@@ -94,12 +94,12 @@ __device__ __forceinline__ void add_rows(const DevScene &sc, const float *out, i
 // accumulators in global memory with coalesced reductions, which the L2 absorbs (about 20 G rows
 // of 64 floats a second): no accumulators shared by the tile's warps, no flush, no barrier.
 // Bound by instruction issue (59 % of the cycles at 12 warps an SM).  Compiled for 3 blocks of 128
-// threads per SM (168 registers): at 4 blocks the pair's state spills (1M rolling-shutter 1080p
+// threads per SM (167 registers): at 4 blocks the pair's state spills (1M rolling-shutter 1080p
 // training step 2558 us against 2520, backward of 200k particles at 640x480 890 against 780), at 5
 // far more.  Against one pixel a thread with accumulators shared by the tile's warps: that step
 // 3058 -> 2449 us, that backward 1143 -> 718 us, the 8-view step of 3M particles 58.9 -> 46.3 ms
 // (with the forward's change); with one branch a survivor and each reciprocal taken once:
-// 2415 -> 2269, 791 -> 669 us and 46.8 -> 42.4 ms.
+// 2415 -> 2269, 791 -> 669 us and 46.8 -> 42.4 ms.  The scaled reciprocal costs 0.8 % (that backward).
 // PP (per-particle colour mode): the colour gradient dL/dc is one 3-vector per particle, summed
 // in the three spare slots of the reduce-scatter; after each round it becomes
 // dL/dbeta = dL/dc Y(dir) and the mean's gradient through the view direction.

@@ -39,9 +39,9 @@ __device__ __forceinline__ void store_pixel(const DevView &view, const DevCam &c
 constexpr int fwd_blocks(int deg, bool rs, bool pp) { return pp ? (rs ? 6 : 8) : (deg < 2 ? 6 : 4); }
 
 // Forward compositing, two pixels a thread and 64 a warp (composite_warp.cuh).  Against one pixel a
-// thread with the block's shared staging: 1M rolling-shutter 1080p, this kernel alone, 578 M -> 348 M
-// warp instructions, 616 -> 470 us (issue 58 %, FMA pipe 56 % of the cycles at 16 warps an SM: bound
-// by both); composite_forward of 200k particles at 3840x2160 977 -> 806 us; 8 views of 3M particles
+// thread with the block's shared staging: 1M rolling-shutter 1080p, this kernel alone, 578 M -> 337 M
+// warp instructions, 616 -> 459 us (issue 60 %, FMA pipe 59 % of the cycles at 16 warps an SM: bound
+// by both); composite_forward of 200k particles at 3840x2160 964 -> 768 us; 8 views of 3M particles
 // 13.4 -> 11 ms; the image is bit-identical.
 // PP: per-particle colour mode (the colour of each staged particle is evaluated once, at its
 // view direction, while staging; pixels read it from shared memory).
